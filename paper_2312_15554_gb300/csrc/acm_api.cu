@@ -1403,7 +1403,7 @@ acm_status ctx_create(acm_ctx** out, int n0, int n1, int n2, void* stream, int B
   g.us = 3 * g.V;
   g.lph = 1;
   c->st = (cudaStream_t)stream;
-  const int nbx = Ops<float>::x_blocks(g);
+  const int nbx = std::max(Ops<float>::x_blocks(g), Ops<double>::x_blocks(g));
   // partial sums sized for the narrowest tile variant the autotuner may pick
   Geo gn = g;
   for (int pr = 0; pr < 2; ++pr)

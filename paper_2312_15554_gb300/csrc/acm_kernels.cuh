@@ -131,26 +131,50 @@ __device__ __forceinline__ void x_fft(cx<T>* sm, const cx<T>* tw) {
 }
 
 // ---------------------------------------------------------------------------
-// Line-resident x passes (acm_xline.cuh): blocks of XS_WARPS warps, each warp
-// taking XS_GPW consecutive groups of LPW lines.
+// Line-resident x passes (acm_xline.cuh): blocks of up to XS_WARPS warps, each
+// warp taking gpw consecutive groups of LPW lines.
 // ---------------------------------------------------------------------------
-constexpr int XS_WARPS = 8;   // warps per block of the line-resident x passes
-constexpr int XS_GPW = 4;     // line groups per warp
+constexpr int XS_WARPS = 8;   // most warps per block of the line-resident x passes
+constexpr int XS_GPW = 4;     // line groups per warp on large grids
 constexpr int XS_PCACHE = 4;  // solute x pass: problems whose parameters a block converts once
 
 template <typename T, int N2>
-__host__ __device__ constexpr int xs_tw_slots() { return (tw_total(N2 / 2) + N2 / 2 + 1 + 1) / 2 * 2; }
+__host__ __device__ constexpr int xs_tw_slots() { return (XL<T, N2>::TW + 1) / 2 * 2; }
 
-// shared memory: twiddles, NBUF line buffers per line, and ACC real values per lane
+// shared memory of a block of `warps`: twiddles, NBUF line buffers per line, and
+// ACC real values per lane
 template <typename T, int N2, int NBUF, int ACC>
-__host__ __device__ constexpr int xs_smem_bytes() {
-  return (xs_tw_slots<T, N2>() + XS_WARPS * XL<T, N2>::LPW * XL<T, N2>::template lb<NBUF>()) * (int)sizeof(cx<T>) +
-         XS_WARPS * 32 * ACC * (int)sizeof(T);
+__host__ __device__ constexpr int xs_smem_bytes(int warps = XS_WARPS) {
+  return (xs_tw_slots<T, N2>() + warps * XL<T, N2>::LPW * XL<T, N2>::template lb<NBUF>()) * (int)sizeof(cx<T>) +
+         warps * 32 * ACC * (int)sizeof(T);
 }
 
-// blocks per problem of the line-resident x passes
-__host__ __device__ constexpr int xs_blocks(int lines, int lpw) {
-  return (lines / lpw + XS_WARPS * XS_GPW - 1) / (XS_WARPS * XS_GPW);
+// Launch shape of a line-resident x pass over `groups` line groups of one
+// problem. Grids that give two blocks of eight warps with four groups each to
+// every SM (152) take that shape, whose warps prefetch their next group;
+// smaller grids take one group per warp and halve the block until there are two
+// blocks per SM (or one warp a block); below four warps a block the three
+// components, which the Stokes passes treat one by one, go to blocks of their own
+// (csplit = 3, blockIdx.z). The shape depends on the grid alone, so the partial
+// sums of a problem do not depend on how many share its launch. Below about
+// 10000 groups a pass is latency-bound: with four groups per warp everywhere the
+// 32^3 FP64 x passes ran in one block (585 and 403 us a launch, now 14 and 10),
+// 64^3 FP32 in eight (71 and 41, now 11 and 7.6), the 128^3 solute pass in 64
+// (59, now 30), and a 128 x 128 plane in one (42 and 25, now 8.7 and 6.3).
+struct XGrid {
+  int warps, gpw, blocks, csplit;
+};
+
+__host__ constexpr XGrid xs_grid(int groups) {
+  constexpr int WANT = 304;
+  XGrid x{XS_WARPS, XS_GPW, 0, 1};
+  if (groups < XS_WARPS * XS_GPW * WANT) {
+    x.gpw = 1;
+    while (x.warps > 1 && groups < x.warps * WANT) x.warps /= 2;
+    if (x.warps < 4) x.csplit = 3;
+  }
+  x.blocks = (groups + x.warps * x.gpw - 1) / (x.warps * x.gpw);
+  return x;
 }
 
 // ---------------------------------------------------------------------------
@@ -165,7 +189,7 @@ template <typename T, int N2>
 __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     k_x_stokes_local(const cx<T>* __restrict__ spec, T* __restrict__ u, T* __restrict__ lam,
                      const uint8_t* __restrict__ H, const uint32_t* __restrict__ Hb, StokesDev* __restrict__ prm,
-                     double* __restrict__ part, Geo g, const cx<T>* __restrict__ twg) {
+                     double* __restrict__ part, Geo g, const cx<T>* __restrict__ twg, int gpw) {
   using L = XL<T, N2>;
   constexpr int M = L::M, E = L::E, TL = L::TL, LPW = L::LPW, LS = L::LS;
   constexpr int LB = L::template lb<2>();
@@ -177,9 +201,11 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   __shared__ T red[5 * 32];
   __shared__ T kpar[3];
   const int p = blockIdx.y;
+  // components of this block: all three, or one each (see xs_grid)
+  const int cb = blockIdx.z, ce = gridDim.z == 1 ? 3 : cb + 1;
   StokesDev* P = prm + p;
   if (P->done) return;
-  load_tw_x<T, N2>(tw, twg);
+  xl_load_tw<T, N2, TW_MAX>(tw, twg);
   if (threadIdx.x == 0) {
     // penalties in the kernel's precision, converted once per block;
     // u~^n on solid voxels = s_prev u^n (s_prev = 1 before the first iteration)
@@ -205,9 +231,9 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   // residual partials of the lane over all its lines, in T (a few hundred terms)
   T d5[5] = {0, 0, 0, 0, 0};
   const int ngroups = g.n0 * g.n1 / LPW;
-  const int gbase = (blockIdx.x * XS_WARPS + warp) * XS_GPW;
+  const int gbase = (blockIdx.x * (blockDim.x >> 5) + warp) * gpw;
 #pragma unroll 1
-  for (int gi = 0; gi < XS_GPW; ++gi) {
+  for (int gi = 0; gi < gpw; ++gi) {
     const int grp = gbase + gi;
     if (grp >= ngroups) break;
     const long long line = (long long)grp * LPW + ll;
@@ -215,8 +241,8 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     const cx<T>* srow = sp + line * g.P;
     __syncwarp(mask);
     for (int e = t; e <= M; e += TL) {
-      cp_async<(int)sizeof(cx<T>)>(&b0[pad(e)], &srow[e]);
-      cp_async<(int)sizeof(cx<T>)>(&b1[pad(e)], &srow[g.S + e]);
+      cp_async<(int)sizeof(cx<T>)>(&b0[pad(e)], &srow[cb * g.S + e]);
+      if (ce > cb + 1) cp_async<(int)sizeof(cx<T>)>(&b1[pad(e)], &srow[(cb + 1) * g.S + e]);
     }
     cp_async_commit();
     if (lane == 0) {
@@ -225,12 +251,10 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
       // voxels only and is left to the predicated loads
       const long long w0 = (long long)grp * LPW * N2;
       constexpr unsigned RB = LPW * N2 * sizeof(T);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) prefetch_l2(up + c * g.V + w0, RB);
-      if (gi + 1 < XS_GPW && grp + 1 < ngroups) {
+      for (int c = cb; c < ce; ++c) prefetch_l2(up + c * g.V + w0, RB);
+      if (gi + 1 < gpw && grp + 1 < ngroups) {
         const unsigned SB = (unsigned)(LPW * g.P * sizeof(cx<T>));
-#pragma unroll
-        for (int c = 0; c < 3; ++c) prefetch_l2(sp + c * g.S + (long long)(grp + 1) * LPW * g.P, SB);
+        for (int c = cb; c < ce; ++c) prefetch_l2(sp + c * g.S + (long long)(grp + 1) * LPW * g.P, SB);
       }
     }
     const unsigned hm = xl_hmask<N2, TL, E>(Hbp, Hp, line, t);
@@ -240,8 +264,8 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     cx<T> v[E];
     static_assert(E % CH == 0, "whole chunks per component");
 #pragma unroll 1
-    for (int c = 0; c < 3; ++c) {
-      cx<T>* bc = c == 1 ? b1 : b0;
+    for (int c = cb; c < ce; ++c) {
+      cx<T>* bc = c == cb + 1 ? b1 : b0;
       T* uc = up + c * g.V + v0;
       T* lc = lp + c * g.V + v0;
       // old state of the component: the first chunk travels during the inverse
@@ -298,7 +322,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
       };
       load_chunk(0, ua, la);
       xl_inverse<T, N2>(bc, tw, t, mask, v);
-      if (c == 0) {
+      if (c == cb && ce == cb + 3) {
         // the row of component 2 into b0, behind components 0 and 1
         __syncwarp(mask);
         for (int e = t; e <= M; e += TL) cp_async<(int)sizeof(cx<T>)>(&b0[pad(e)], &srow[2 * g.S + e]);
@@ -314,7 +338,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
         if (j & 1) step_chunk(j * CH, ub, lb);
         else step_chunk(j * CH, ua, la);
       }
-      if (c == 1) {
+      if (c == cb + 1) {
         cp_async_wait<0>();
         __syncwarp(mask);
       }
@@ -325,7 +349,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     d5[3] += a3;
     d5[4] += a4;
   }
-  block_sum_store<5>(d5, red, part + ((long long)p * gridDim.x + blockIdx.x) * 8);
+  block_sum_store<5>(d5, red, part + (((long long)p * gridDim.z + blockIdx.z) * gridDim.x + blockIdx.x) * 8);
 }
 
 // ---------------------------------------------------------------------------
@@ -335,7 +359,7 @@ template <typename T, int N2>
 __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     k_x_stokes_rhs(cx<T>* __restrict__ spec, const T* __restrict__ u, const T* __restrict__ lam,
                    const uint8_t* __restrict__ H, const uint32_t* __restrict__ Hb, const StokesDev* __restrict__ prm,
-                   Geo g, const cx<T>* __restrict__ twg) {
+                   Geo g, const cx<T>* __restrict__ twg, int gpw) {
   using L = XL<T, N2>;
   constexpr int M = L::M, E = L::E, TL = L::TL, LPW = L::LPW;
   constexpr int LB = L::template lb<1>();
@@ -346,9 +370,11 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   cx<T>* lines = tw + xs_tw_slots<T, N2>();
   __shared__ T kpar[2];
   const int p = blockIdx.y;
+  // components of this block: all three, or one each (see xs_grid)
+  const int cb = blockIdx.z, ce = gridDim.z == 1 ? 3 : cb + 1;
   const StokesDev* P = prm + p;
   if (P->done) return;
-  load_tw_x<T, N2>(tw, twg);
+  xl_load_tw<T, N2, TW_MAX>(tw, twg);
   if (threadIdx.x == 0) {
     // converted once per block; u~^n on solid voxels = s_prev u^n with the
     // penalties of the iteration just taken
@@ -367,9 +393,9 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   const T* lp = lam + (long long)p * 3 * g.V;
   const long long hcell = (long long)(p / g.lph) * g.hs;
   const int ngroups = g.n0 * g.n1 / LPW;
-  const int gbase = (blockIdx.x * XS_WARPS + warp) * XS_GPW;
+  const int gbase = (blockIdx.x * (blockDim.x >> 5) + warp) * gpw;
 #pragma unroll 1
-  for (int gi = 0; gi < XS_GPW; ++gi) {
+  for (int gi = 0; gi < gpw; ++gi) {
     const int grp = gbase + gi;
     if (grp >= ngroups) break;
     const long long line = (long long)grp * LPW + ll;
@@ -377,7 +403,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     const unsigned hm = xl_hmask<N2, TL, E>(Hb + hcell / 32, H + hcell, line, t);
     cx<T> v[E];
 #pragma unroll 1
-    for (int c = 0; c < 3; ++c) {
+    for (int c = cb; c < ce; ++c) {
       // Eq. 7 right-hand side w = b u~ - a with a = H lambda (the Green step adds g and -i d q)
       const T* uc = up + c * g.V + v0;
       const T* lc = lp + c * g.V + v0;
@@ -432,7 +458,7 @@ template <typename T, int N2, bool CEN>
 __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     k_x_solute(cx<T>* __restrict__ spec, const T* __restrict__ u, const uint8_t* __restrict__ H,
                const uint32_t* __restrict__ Hb, const SoluteDev* __restrict__ prm, Geo g,
-               const cx<T>* __restrict__ twg, const T* __restrict__ d2, int nprob, int gpw) {
+               const cx<T>* __restrict__ twg, const T* __restrict__ d2, int nprob, int gpw, int pshare) {
   using L = XL<T, N2>;
   constexpr int M = L::M, E = L::E, TL = L::TL, LPW = L::LPW, LS = L::LS;
   constexpr int LB = L::template lb<2>();
@@ -441,18 +467,17 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   cx<T>* tw = reinterpret_cast<cx<T>*>(smem_raw);
   cx<T>* lines = tw + xs_tw_slots<T, N2>();
   // s accumulated per lane as voxel pairs: [m][lane] for conflict-free access
-  T2* acc = reinterpret_cast<T2*>(lines + XS_WARPS * LPW * LB) + (threadIdx.x >> 5) * 32 * E;
+  T2* acc = reinterpret_cast<T2*>(lines + (blockDim.x >> 5) * LPW * LB) + (threadIdx.x >> 5) * 32 * E;
   // Problems that share one velocity and indicator (us = hs = 0, e.g. the three
-  // composition loads of a tensor solve) run back to back on the same warp, so
-  // each velocity row crosses DRAM once (up to XS_PCACHE problems per block,
-  // blockIdx.y numbering the groups); otherwise blockIdx.y is the problem.
-  const bool shared = g.us == 0 && g.hs == 0;
-  const int pbeg = shared ? blockIdx.y * XS_PCACHE : blockIdx.y;
-  const int pend = shared ? min(nprob, pbeg + XS_PCACHE) : blockIdx.y + 1;
+  // composition loads of a tensor solve) run back to back on the same warp on
+  // large grids, so each velocity row crosses DRAM once: pshare (1 ..
+  // XS_PCACHE) problems per block, blockIdx.y numbering the groups.
+  const int pbeg = blockIdx.y * pshare;
+  const int pend = min(nprob, pbeg + pshare);
   bool any = false;
   for (int p = pbeg; p < pend; ++p) any = any || !prm[p].done;
   if (!any) return;
-  load_tw_x<T, N2>(tw, twg);
+  xl_load_tw<T, N2, TW_MAX>(tw, twg);
   // parameters of the block's problems in T, converted once per block:
   // (g_c, B0_c) for c = 0..2, then A0, eta, Pe, Fc
   __shared__ T spar[XS_PCACHE][10];
@@ -474,7 +499,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   cx<T>* b0 = lines + (warp * LPW + ll) * LB;
   cx<T>* b1 = b0 + LS;
   const int ngroups = g.n0 * g.n1 / LPW;
-  const int gbase = (blockIdx.x * XS_WARPS + warp) * gpw;
+  const int gbase = (blockIdx.x * (blockDim.x >> 5) + warp) * gpw;
 #pragma unroll 1
   for (int gi = 0; gi < gpw; ++gi) {
     const int grp = gbase + gi;
@@ -638,7 +663,8 @@ __global__ void __launch_bounds__(NC * 64) k_x_r2c(cx<T>* __restrict__ spec, con
 template <typename T, int N2>
 __global__ void __launch_bounds__(XS_WARPS * 32) k_x_c2r_lr(const cx<T>* __restrict__ spec, T* __restrict__ out,
                                                            Geo g, int nc, long long outProbStride,
-                                                           long long specProbStride, const cx<T>* __restrict__ twg) {
+                                                           long long specProbStride, const cx<T>* __restrict__ twg,
+                                                           int gpw) {
   using L = XL<T, N2>;
   constexpr int M = L::M, E = L::E, TL = L::TL, LPW = L::LPW;
   constexpr int LB = L::template lb<1>();
@@ -647,7 +673,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32) k_x_c2r_lr(const cx<T>* __restr
   cx<T>* tw = reinterpret_cast<cx<T>*>(smem_raw);
   cx<T>* lines = tw + xs_tw_slots<T, N2>();
   const int p = blockIdx.y / nc, c = blockIdx.y % nc;
-  load_tw_x<T, N2>(tw, twg);
+  xl_load_tw<T, N2, TW_MAX>(tw, twg);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ll = lane / TL, t = lane % TL;
@@ -656,9 +682,9 @@ __global__ void __launch_bounds__(XS_WARPS * 32) k_x_c2r_lr(const cx<T>* __restr
   const cx<T>* sp = spec + p * specProbStride + c * g.S;
   T* op = out + p * outProbStride + c * g.V;
   const int ngroups = g.n0 * g.n1 / LPW;
-  const int gbase = (blockIdx.x * XS_WARPS + warp) * XS_GPW;
+  const int gbase = (blockIdx.x * (blockDim.x >> 5) + warp) * gpw;
 #pragma unroll 1
-  for (int gi = 0; gi < XS_GPW; ++gi) {
+  for (int gi = 0; gi < gpw; ++gi) {
     const int grp = gbase + gi;
     if (grp >= ngroups) break;
     const long long line = (long long)grp * LPW + ll;

@@ -57,9 +57,9 @@ static cudaError_t l_x_local(const Geo& g, int nprob, const void* spec, void* u,
   constexpr int smem = xs_smem_bytes<T, N2, 2, 0>();
   static const cudaError_t attr = set_smem(k_x_stokes_local<T, N2>, smem);
   if (attr != cudaSuccess) return attr;
-  dim3 grid(xs_blocks(g.n0 * g.n1, XL<T, N2>::LPW), nprob);
-  k_x_stokes_local<T, N2><<<grid, XS_WARPS * 32, smem, s>>>((const cx<T>*)spec, (T*)u, (T*)lam, H, Hb, prm, part, g,
-                                                            (const cx<T>*)tw);
+  const XGrid x = xs_grid(g.n0 * g.n1 / XL<T, N2>::LPW);
+  k_x_stokes_local<T, N2><<<dim3(x.blocks, nprob, x.csplit), x.warps * 32, xs_smem_bytes<T, N2, 2, 0>(x.warps), s>>>(
+      (const cx<T>*)spec, (T*)u, (T*)lam, H, Hb, prm, part, g, (const cx<T>*)tw, x.gpw);
   return cudaGetLastError();
 }
 
@@ -69,9 +69,9 @@ static cudaError_t l_x_rhs(const Geo& g, int nprob, void* spec, const void* u, c
   constexpr int smem = xs_smem_bytes<T, N2, 1, 0>();
   static const cudaError_t attr = set_smem(k_x_stokes_rhs<T, N2>, smem);
   if (attr != cudaSuccess) return attr;
-  dim3 grid(xs_blocks(g.n0 * g.n1, XL<T, N2>::LPW), nprob);
-  k_x_stokes_rhs<T, N2><<<grid, XS_WARPS * 32, smem, s>>>((cx<T>*)spec, (const T*)u, (const T*)lam, H, Hb, prm, g,
-                                                          (const cx<T>*)tw);
+  const XGrid x = xs_grid(g.n0 * g.n1 / XL<T, N2>::LPW);
+  k_x_stokes_rhs<T, N2><<<dim3(x.blocks, nprob, x.csplit), x.warps * 32, xs_smem_bytes<T, N2, 1, 0>(x.warps), s>>>(
+      (cx<T>*)spec, (const T*)u, (const T*)lam, H, Hb, prm, g, (const cx<T>*)tw, x.gpw);
   return cudaGetLastError();
 }
 
@@ -84,20 +84,21 @@ static cudaError_t l_x_solute(const Geo& g, int nprob, void* spec, const void* u
   static const cudaError_t attr1 = set_smem(k_x_solute<T, N2, true>, smem);
   if (attr0 != cudaSuccess) return attr0;
   if (attr1 != cudaSuccess) return attr1;
-  // problems sharing the velocity and the indicator loop inside the kernel (up
-  // to XS_PCACHE per block), with fewer line groups per warp so that the grid
-  // keeps its size
-  const bool shared = g.us == 0 && g.hs == 0;
-  const int np_blk = nprob < XS_PCACHE ? nprob : XS_PCACHE;
-  const int gpw = shared ? (XS_GPW / np_blk > 1 ? XS_GPW / np_blk : 1) : XS_GPW;
-  const int ngroups = g.n0 * g.n1 / XL<T, N2>::LPW;
-  dim3 grid((ngroups + XS_WARPS * gpw - 1) / (XS_WARPS * gpw), shared ? (nprob + XS_PCACHE - 1) / XS_PCACHE : nprob);
-  if (central)
-    k_x_solute<T, N2, true><<<grid, XS_WARPS * 32, smem, s>>>((cx<T>*)spec, (const T*)u, H, Hb, prm, g,
-                                                               (const cx<T>*)tw, d2, nprob, gpw);
-  else
-    k_x_solute<T, N2, false><<<grid, XS_WARPS * 32, smem, s>>>((cx<T>*)spec, (const T*)u, H, Hb, prm, g,
-                                                                (const cx<T>*)tw, d2, nprob, gpw);
+  // On grids large enough for gpw > 1, problems that share the velocity and the
+  // indicator loop inside the kernel (up to XS_PCACHE per block), with fewer line
+  // groups per warp so that the grid keeps its size. On smaller ones the velocity
+  // stays in L2 and each problem gets blocks of its own.
+  XGrid x = xs_grid(g.n0 * g.n1 / XL<T, N2>::LPW);
+  int pshare = 1;
+  if (g.us == 0 && g.hs == 0 && x.gpw > 1) {
+    pshare = nprob < XS_PCACHE ? nprob : XS_PCACHE;
+    x.gpw = XS_GPW / pshare > 1 ? XS_GPW / pshare : 1;
+    x.blocks = (g.n0 * g.n1 / XL<T, N2>::LPW + x.warps * x.gpw - 1) / (x.warps * x.gpw);
+  }
+  const dim3 grid(x.blocks, (nprob + pshare - 1) / pshare);
+  auto* k = central ? k_x_solute<T, N2, true> : k_x_solute<T, N2, false>;
+  k<<<grid, x.warps * 32, xs_smem_bytes<T, N2, 2, 2 * XL<T, N2>::E>(x.warps), s>>>(
+      (cx<T>*)spec, (const T*)u, H, Hb, prm, g, (const cx<T>*)tw, d2, nprob, x.gpw, pshare);
   return cudaGetLastError();
 }
 
@@ -139,9 +140,9 @@ static cudaError_t l_x_c2r(const Geo& g, int nprob, int nc, const void* spec, lo
     constexpr int smem = xs_smem_bytes<T, N2, 1, 0>();
     static const cudaError_t attr = set_smem(k_x_c2r_lr<T, N2>, smem);
     if (attr != cudaSuccess) return attr;
-    dim3 grid(xs_blocks(g.n0 * g.n1, XL<T, N2>::LPW), nprob * nc);
-    k_x_c2r_lr<T, N2><<<grid, XS_WARPS * 32, smem, s>>>((const cx<T>*)spec, (T*)out, g, nc, ops, sps,
-                                                        (const cx<T>*)tw);
+    const XGrid x = xs_grid(g.n0 * g.n1 / XL<T, N2>::LPW);
+    k_x_c2r_lr<T, N2><<<dim3(x.blocks, nprob * nc), x.warps * 32, xs_smem_bytes<T, N2, 1, 0>(x.warps), s>>>(
+        (const cx<T>*)spec, (T*)out, g, nc, ops, sps, (const cx<T>*)tw, x.gpw);
     return cudaGetLastError();
   }
   if (nc == 1) return l_x_c2r_nc<T, N2, 1>(g, nprob, spec, sps, out, ops, tw, s);
@@ -331,8 +332,9 @@ static cudaError_t l_pass(const Geo& g, int axis, int op, int nc, int nprob, voi
 template <typename T>
 int Ops<T>::x_blocks(const Geo& g) {
   const int M = g.n2 / 2;
-  const int TL = M / ept(M);
-  return xs_blocks(g.n0 * g.n1, 32 / TL);
+  const int TL = M / xl_ept<T>(M);
+  const XGrid x = xs_grid(g.n0 * g.n1 / (32 / TL));
+  return x.blocks * x.csplit;
 }
 
 template <typename T>

@@ -6,8 +6,8 @@
 // a warp own one line; lane t of the line holds the E elements
 // z[t + TL m], m = 0..E-1, in registers.
 //
-// With E = 16 and TL > 1 the transform has two Stockham stages (radix E, then
-// radix TL). The first stage reads exactly the elements t + TL m of its own
+// With TL > 1 the transform has two Stockham stages (radix E, then radix
+// TL <= E). The first stage reads exactly the elements t + TL m of its own
 // lane, and the second stage leaves its lane with exactly those positions too,
 // so between an inverse and a forward transform the local step of the method
 // runs on registers, and the voxels 2k, 2k+1 (k = t + TL m) of every component
@@ -21,13 +21,26 @@
 
 namespace acm {
 
+// Elements per lane. FP32 lanes take up to 16. FP64 lines shorter than 256
+// voxels take the most even split M = E x TL: the FP64 pipe of an SM runs two
+// multiply-adds a cycle, so an FP64 pass on a small grid is bound by how many SMs
+// have warps, and a 32-voxel line on four lanes of four elements gives four
+// times the warps of one lane of 16.
+template <typename T>
+__host__ __device__ constexpr int xl_ept(int M) {
+  return sizeof(T) == 8 ? (M >= 128 ? 16 : (M >= 32 ? 8 : 4)) : ept(M);
+}
+
 template <typename T, int N2>
 struct XL {
   static constexpr int M = N2 / 2;
-  static constexpr int E = ept(M);
+  static constexpr int E = xl_ept<T>(M);
   static constexpr int TL = M / E;        // lanes per line
   static constexpr int LPW = 32 / TL;     // lines per warp
   static constexpr int NB = E / TL;       // second-stage groups per lane (TL > 1)
+  static_assert(TL <= E && E * TL == M, "two stages: radix E, then radix TL");
+  // twiddle table of a block: W_N2^t (t < TL), then W_M^{t r} at TL r + t (r = 1..TL-1)
+  static constexpr int TW = TL * TL;
   // slots per line buffer: X[0..M] (pad(M) included), bank-friendly for TL lanes
   static constexpr int LS = line_stride(M + 1, TL, 0, wave_slots<T>());
   // stride between the consecutive lines of a warp holding NBUF buffers each:
@@ -42,6 +55,16 @@ struct XL {
     return s;
   }
 };
+
+// The table of XL::TW twiddles from W_TWM^k, k < TWM (TWM a multiple of 2 N2).
+template <typename T, int N2, int TWM>
+__device__ __forceinline__ void xl_load_tw(cx<T>* tw, const cx<T>* __restrict__ master) {
+  using L = XL<T, N2>;
+  for (int e = threadIdx.x; e < L::TW; e += blockDim.x) {
+    const int r = e / L::TL, t = e - r * L::TL;
+    tw[e] = master[r == 0 ? t * (TWM / N2) : ((t * r) % L::M) * (TWM / L::M)];
+  }
+}
 
 // Indicator bits of the lane's voxels 2k, 2k+1 (k = t + TL m) as bits 2m, 2m+1.
 // Hb: one bit per voxel, 32 voxels per word in index order (lines of N2 >= 32
@@ -99,12 +122,11 @@ __device__ __forceinline__ cx<T> xl_post(cx<T> Zk, cx<T> Zm, cx<T> wt) {
 template <typename T, int N2, int SIGN>
 __device__ __forceinline__ void xl_stage2(const cx<T>* sl, const cx<T>* tw, int t, cx<T> (&v)[XL<T, N2>::E]) {
   using L = XL<T, N2>;
-  constexpr int M = L::M, E = L::E, TL = L::TL, NB = L::NB;
+  constexpr int E = L::E, TL = L::TL, NB = L::NB;
   cx<T> w0[TL];
-  const cx<T>* tws = tw + tw_offset(M, E) + t;
 #pragma unroll
   for (int r = 1; r < TL; ++r) {
-    w0[r] = tws[(r - 1) * E];
+    w0[r] = tw[r * TL + t];
     if constexpr (SIGN > 0) w0[r].y = -w0[r].y;
   }
   static_for<NB>([&](auto I) {
@@ -131,7 +153,7 @@ __device__ __forceinline__ void xl_inverse(cx<T>* sl, const cx<T>* tw, int t, un
                                            cx<T> (&v)[XL<T, N2>::E]) {
   using L = XL<T, N2>;
   constexpr int M = L::M, E = L::E, TL = L::TL;
-  const cx<T> wt = tw[tw_total(M) + t];
+  const cx<T> wt = tw[t];
   static_for<E>([&](auto R) {
     constexpr int r = decltype(R)::value;
     const int k = t + TL * r;
@@ -165,7 +187,7 @@ __device__ __forceinline__ void xl_forward(cx<T>* sl, const cx<T>* tw, int t, un
   using L = XL<T, N2>;
   constexpr int M = L::M, E = L::E, TL = L::TL;
   static_assert(E % 2 == 0, "positions finish in pairs");
-  const cx<T> wt = tw[tw_total(M) + t];
+  const cx<T> wt = tw[t];
   dft<E, -1>(v);
   __syncwarp(mask);  // earlier readers of sl are done
 #pragma unroll

@@ -245,15 +245,21 @@ acm_status acm_batch_stokes(acm_batch* batch, const uint8_t* const* H, const acm
                             void* const* lambda_out, double* K, acm_report* rep);
 /* Tile autotuner. The strided FFT passes of the solver loops (y forward and
  * inverse of the Stokes iteration, the z pass with the Green step of Eq. 13,
- * the y forward, z pass (Eq. 20) and y inverse of the solute iteration) exist in up to
- * three tile widths (columns per block). acm_autotune times each candidate on
- * the context's workspace and stream and keeps the fastest for that precision
- * (fp64 0/1) and derivative symbol; acm_batch_autotune does so per cell shape
- * with the batch's problem count. Fields do not depend on the choice; only the
- * summation order of the FP64 residual partials does. tiles (out, nullable):
- * the widths in the order y-forward Stokes, z Stokes, y-inverse Stokes,
- * y-forward solute, z solute, y-inverse solute (0 where a pass does not apply). acm_set_tiles sets them explicitly
- * (ACM_ERR_ARG for a width that has no compiled variant); acm_get_tiles reads
+ * the y forward, z pass (Eq. 20) and y inverse of the solute iteration) exist in
+ * several tile widths (columns per block). Left alone, a pass picks its width from
+ * the grid. acm_autotune times the candidates on the context's workspace and stream
+ * and keeps the fastest for that precision (fp64 0/1) and derivative symbol;
+ * acm_batch_autotune does so per cell shape with the batch's problem count. The
+ * candidates of one pass give the same fields bit for bit; only the summation order
+ * of the residual partials differs. tiles (out, nullable): the widths in the
+ * order y-forward Stokes, z Stokes, y-inverse Stokes, y-forward solute, z solute,
+ * y-inverse solute (0 where a pass does not apply). At 64, 128 and 256 points the
+ * tuner's candidates are row segments of 128 and 64 bytes, reported as negative
+ * widths (FP32 -16 and -8, FP64 -8 and -4), except in the z solute pass; in FP32 they
+ * round differently from the positive widths (about 1e-7 of a field).
+ * acm_set_tiles sets widths explicitly (ACM_ERR_ARG for one outside the set that
+ * the pass offers); a pass runs the nearest width that is compiled for its line
+ * length, and the default width leaves the choice to the grid. acm_get_tiles reads
  * the current widths. Call between solves. */
 acm_status acm_autotune(acm_ctx* ctx, int fp64, int deriv, int tiles[6]);
 acm_status acm_set_tiles(acm_ctx* ctx, int fp64, const int tiles[6]);

@@ -872,7 +872,7 @@ acm_status solute_body(acm_ctx* c, int nprob, const uint8_t* Hdev, const void* u
   const int nbz = Ops<T>::z_blocks(g, P_SOLUTE);
   const long long ps = 4 * g.S;
   // spectral components per problem: x -> (tau_0, tau_1, s + d2 tau_2), y forward -> (tau_0, s''),
-  // z -> (d0 chi, chi), y inverse -> (d0 chi, d1 chi, d2 chi)
+  // z -> (d0 chi, -, -, chi), y inverse -> (d0 chi, d1 chi, d2 chi)
   LK(ACM_K_X_SOLUTE, Ops<T>::x_solute(g, nprob, w.spec, udev, Hdev, c->Hb, c->cprm, w.tw, sym,
                                      c->solute_deriv == ACM_DERIV_CENTRAL, c->st));
   LK(ACM_K_Y_FWD_SOLUTE, Ops<T>::pass(g, 1, P_FWD_SOL, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, nullptr, c->cprm,
@@ -1326,11 +1326,16 @@ acm_status autotune_ctx(acm_ctx* c, int nprob, int deriv) {
     const int n = j.axis == 1 ? c->g.n1 : c->g.n0;
     float best = 0;
     int best_sh = 0;
-    for (int sh = -1; sh <= 4 && st == ACM_OK; ++sh) {   // 3, 4: the register-resident variants
+    // Where the row-segment widths (3, 4) exist they are the candidates, except for
+    // the solute z pass, which takes the others: the choices of either set agree bit
+    // for bit, so a tuned context's results do not hang on which of them won.
+    const bool seg = Ops<T>::tx_variant(n, j.op, j.nc, 3);
+    const int first = seg && j.op != P_SOLUTE ? 3 : -1, last = seg && j.op == P_SOLUTE ? 2 : 4;
+    for (int sh = first; sh <= last && st == ACM_OK; ++sh) {
       if (!Ops<T>::tx_variant(n, j.op, j.nc, sh)) continue;
       Geo g = c->g;
       g.txs[pr][j.axis][j.op] = (signed char)sh;
-      const long long ps = (long long)j.nc * g.S;
+      const long long ps = (j.solute ? 4LL : 3LL) * g.S;
       StokesDev* sp = j.solute ? nullptr : c->sprm;
       SoluteDev* cp = j.solute ? c->cprm : nullptr;
       void* s0 = j.op == P_STOKES || j.op == P_SOLUTE ? w.st0 : nullptr;
@@ -1346,11 +1351,9 @@ acm_status autotune_ctx(acm_ctx* c, int nprob, int deriv) {
       if (st == ACM_OK && (cudaEventRecord(e1, c->st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
                            cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess))
         st = ACM_ERR_CUDA;
-      if (st == ACM_OK && (sh == -1 || best == 0 || ms < best)) {
-        if (best == 0 || ms < best) {
-          best = ms;
-          best_sh = sh;
-        }
+      if (st == ACM_OK && (best == 0 || ms < best)) {
+        best = ms;
+        best_sh = sh;
       }
     }
     if (st != ACM_OK) break;
@@ -1404,13 +1407,15 @@ acm_status ctx_create(acm_ctx** out, int n0, int n1, int n2, void* stream, int B
   g.lph = 1;
   c->st = (cudaStream_t)stream;
   const int nbx = std::max(Ops<float>::x_blocks(g), Ops<double>::x_blocks(g));
-  // partial sums sized for the narrowest tile variant the autotuner may pick
-  Geo gn = g;
-  for (int pr = 0; pr < 2; ++pr)
-    for (int ax = 0; ax < 2; ++ax)
-      for (int op = 0; op < 8; ++op) gn.txs[pr][ax][op] = -1;
-  const int nbz = std::max(std::max(Ops<float>::z_blocks(gn, P_STOKES), Ops<float>::z_blocks(gn, P_SOLUTE)),
-                           std::max(Ops<double>::z_blocks(gn, P_STOKES), Ops<double>::z_blocks(gn, P_SOLUTE)));
+  // partial sums sized for the narrowest tile any choice may give
+  int nbz = 0;
+  for (int sh = -1; sh <= 4; ++sh) {
+    Geo gn = g;
+    for (int pr = 0; pr < 2; ++pr)
+      for (int op : {P_STOKES, P_SOLUTE}) gn.txs[pr][0][op] = (signed char)sh;
+    for (int op : {P_STOKES, P_SOLUTE})
+      nbz = std::max(nbz, std::max(Ops<float>::z_blocks(gn, op), Ops<double>::z_blocks(gn, op)));
+  }
   c->nbx = nbx;
   c->nbz = nbz;
   bool ok = cudaMalloc(&c->sprm, (size_t)B * sizeof(StokesDev)) == cudaSuccess &&

@@ -168,11 +168,8 @@ template <int SIGN, typename T>
 __device__ __forceinline__ void dft4(cx<T>* v) { dft4<SIGN>(v[0], v[1], v[2], v[3]); }
 
 template <int SIGN, typename T>
-__device__ __forceinline__ void dft8(cx<T>* v) {
-  cx<T> e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
-  cx<T> o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
-  dft4<SIGN>(e0, e1, e2, e3);
-  dft4<SIGN>(o0, o1, o2, o3);
+__device__ __forceinline__ void dft8_combine(cx<T> e0, cx<T> e1, cx<T> e2, cx<T> e3, cx<T> o0, cx<T> o1, cx<T> o2,
+                                             cx<T> o3, cx<T>* v) {
   o1 = tw16<SIGN, 2>(o1);
   o2 = tw16<SIGN, 4>(o2);
   o3 = tw16<SIGN, 6>(o3);
@@ -187,17 +184,17 @@ __device__ __forceinline__ void dft8(cx<T>* v) {
 }
 
 template <int SIGN, typename T>
-__device__ __forceinline__ void dft16(cx<T>* v) {
-  // n = 4 n1 + n2, k = k1 + 4 k2
-  cx<T> y[4][4];
-#pragma unroll
-  for (int n2 = 0; n2 < 4; ++n2) {
-    y[n2][0] = v[n2];
-    y[n2][1] = v[4 + n2];
-    y[n2][2] = v[8 + n2];
-    y[n2][3] = v[12 + n2];
-    dft4<SIGN>(y[n2][0], y[n2][1], y[n2][2], y[n2][3]);
-  }
+__device__ __forceinline__ void dft8(cx<T>* v) {
+  cx<T> e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
+  cx<T> o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
+  dft4<SIGN>(e0, e1, e2, e3);
+  dft4<SIGN>(o0, o1, o2, o3);
+  dft8_combine<SIGN>(e0, e1, e2, e3, o0, o1, o2, o3, v);
+}
+
+// y[n2][k1]: the four-point DFTs over n1 of n = 4 n1 + n2
+template <int SIGN, typename T>
+__device__ __forceinline__ void dft16_combine(cx<T> (&y)[4][4], cx<T>* v) {
   y[1][1] = tw16<SIGN, 1>(y[1][1]);
   y[1][2] = tw16<SIGN, 2>(y[1][2]);
   y[1][3] = tw16<SIGN, 3>(y[1][3]);
@@ -215,6 +212,50 @@ __device__ __forceinline__ void dft16(cx<T>* v) {
     v[k1 + 4] = b;
     v[k1 + 8] = c;
     v[k1 + 12] = d;
+  }
+}
+
+template <int SIGN, typename T>
+__device__ __forceinline__ void dft16(cx<T>* v) {
+  // n = 4 n1 + n2, k = k1 + 4 k2
+  cx<T> y[4][4];
+#pragma unroll
+  for (int n2 = 0; n2 < 4; ++n2) {
+    y[n2][0] = v[n2];
+    y[n2][1] = v[4 + n2];
+    y[n2][2] = v[8 + n2];
+    y[n2][3] = v[12 + n2];
+    dft4<SIGN>(y[n2][0], y[n2][1], y[n2][2], y[n2][3]);
+  }
+  dft16_combine<SIGN>(y, v);
+}
+
+// The rest of a DFT of radix R = 4, 8 or 16 after its first butterflies
+// s[k] = v[k] + v[k + R/2], q[k] = v[k] - v[k + R/2]
+template <int SIGN, typename T>
+__device__ __forceinline__ void dft4_tail(cx<T> t0, cx<T> t1, cx<T> t2, cx<T> u3, cx<T>& v0, cx<T>& v1, cx<T>& v2,
+                                          cx<T>& v3) {
+  const cx<T> t3 = rot4<SIGN>(u3);
+  v0 = t0 + t2;
+  v2 = t0 - t2;
+  v1 = t1 + t3;
+  v3 = t1 - t3;
+}
+template <int R, int SIGN, typename T>
+__device__ __forceinline__ void dft_tail(const cx<T>* s, const cx<T>* q, cx<T>* v) {
+  if constexpr (R == 4) {
+    dft4_tail<SIGN>(s[0], q[0], s[1], q[1], v[0], v[1], v[2], v[3]);
+  } else if constexpr (R == 8) {
+    cx<T> e0, e1, e2, e3, o0, o1, o2, o3;
+    dft4_tail<SIGN>(s[0], q[0], s[2], q[2], e0, e1, e2, e3);
+    dft4_tail<SIGN>(s[1], q[1], s[3], q[3], o0, o1, o2, o3);
+    dft8_combine<SIGN>(e0, e1, e2, e3, o0, o1, o2, o3, v);
+  } else {
+    cx<T> y[4][4];
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2)
+      dft4_tail<SIGN>(s[n2], q[n2], s[4 + n2], q[4 + n2], y[n2][0], y[n2][1], y[n2][2], y[n2][3]);
+    dft16_combine<SIGN>(y, v);
   }
 }
 

@@ -24,6 +24,7 @@
 #include "acm_fft.cuh"
 #include "acm_xline.cuh"
 #include "acm_types.h"
+#include "acm_rpass.cuh"
 
 namespace acm {
 
@@ -731,298 +732,6 @@ __global__ void __launch_bounds__(NC * 64) k_x_c2r(const cx<T>* __restrict__ spe
 }
 
 // ---------------------------------------------------------------------------
-// strided passes: complex FFTs along y or z on tiles of TX consecutive kx
-// columns, with an optional per-wavevector operator between a forward and an
-// inverse transform (z-pass only).
-// ---------------------------------------------------------------------------
-// OP_FWD_SOL (y forward of the solute iteration): lines (tau_0, tau_1, s') in,
-//   (tau_0, s' + i d1 tau_1) out.
-// OP_SOLUTE (z): (tau_0, s'') in, F^ = s'' + i d0 tau_0, Green step, (i d0 chi^, chi^) out.
-// OP_INV_SOL (y inverse): (a, b) in, lines (a, i d1 b, i d2 b) inverse-transformed out.
-enum { OP_FWD = 0, OP_INV = 1, OP_INV_SCALE = 2, OP_STOKES = 3, OP_SOLUTE = 4, OP_DERIV = 5, OP_FWD_SOL = 6,
-       OP_INV_SOL = 7 };
-
-template <typename T>
-struct PassArgs {
-  cx<T>* spec;
-  long long probStride, compStride, rowStride, outerStride;
-  int Pu;           // used kx columns
-  int n1;           // for wavevector indexing in the z-pass
-  Sym<T> sym;
-  const cx<T>* twg;
-  // operator state
-  cx<T>* st0;       // Stokes: q^ ; solute: chi^
-  cx<T>* st1;       // Stokes: div^ of the previous iteration
-  StokesDev* sprm;
-  SoluteDev* cprm;
-  double* part;     // per-block partial sums (stride 4 doubles)
-  double invV;
-  int nkx;          // n2 / 2 (Nyquist column index)
-  int dm;           // OP_DERIV: axis of the derivative
-  int nouter;       // register-resident passes: pencils along the other strided axis
-};
-
-template <typename T, int N, int OP, int NC, int TX>
-struct SCfg {
-  static constexpr int E = ept(N);
-  static constexpr int TL = N / E;
-  static constexpr int LS = line_stride(N, TL, TX, wave_slots<T>());
-  static constexpr int JOBS = NC * TX;
-  static constexpr int THREADS_ALL = JOBS * TL;
-  static constexpr int ROUNDS = THREADS_ALL > 2048 ? 8 : THREADS_ALL > 1024 ? 4 : THREADS_ALL > 512 ? 2 : 1;
-  // whole warps only: extra threads take no line but help with loads and stores
-  static constexpr int NT = ((THREADS_ALL / ROUNDS) + 31) / 32 * 32;
-  static constexpr int SMEM = (NC * TX * LS + tw_total(N)) * (int)sizeof(cx<T>);
-};
-
-// Transforms the tile's lines (line = component * TX + column); lines of the
-// columns w..TX-1 that a tile at the end of a pencil leaves empty are skipped.
-template <typename T, int N, int OP, int NC, int TX, int SIGN, int NLINES>
-__device__ __forceinline__ void s_fft(cx<T>* sm, const cx<T>* tw, int w) {
-  using C = SCfg<T, N, OP, NC, TX>;
-  constexpr int per_round = C::NT / C::TL;
-#pragma unroll 1
-  for (int r = 0; r < C::ROUNDS; ++r) {
-    const int job = r * per_round + threadIdx.x / C::TL;
-    const bool live = job < NLINES && job % TX < w;
-    const unsigned mask = __ballot_sync(0xffffffffu, live);
-    if (live) fft_line<T, N, SIGN>(sm + job * C::LS, threadIdx.x % C::TL, tw, mask);
-  }
-}
-
-template <typename T, int N, int OP, int NC, int TX>
-__global__ void __launch_bounds__(SCfg<T, N, OP, NC, TX>::NT) k_strided(PassArgs<T> a) {
-  using C = SCfg<T, N, OP, NC, TX>;
-  constexpr int NIN = (OP == OP_INV_SOL) ? 2 : NC;
-  constexpr int NOUT = (OP == OP_FWD_SOL) ? 2 : NC;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
-  cx<T>* tw = sm + NC * TX * C::LS;
-  __shared__ T red[4 * 32];
-  // the operator's parameters, converted once per block: (nu, beta, b) or
-  // (A0, B0), and 1/V
-  __shared__ T opar[5];
-  const int p = blockIdx.z, outer = blockIdx.y, kx0 = blockIdx.x * TX;
-  if (a.sprm && a.sprm[p].done) return;
-  if (a.cprm && a.cprm[p].done) return;
-  if constexpr (OP == OP_STOKES) {
-    if (threadIdx.x == 0) {
-      opar[0] = (T)a.sprm[p].nu;
-      opar[1] = (T)a.sprm[p].psi[1];
-      opar[2] = (T)a.sprm[p].psi[2];
-      opar[4] = (T)a.invV;
-    }
-  } else if constexpr (OP == OP_SOLUTE) {
-    if (threadIdx.x == 0) {
-      opar[0] = (T)a.cprm[p].A0;
-      for (int k = 0; k < 3; ++k) opar[1 + k] = (T)a.cprm[p].B0[k];
-      opar[4] = (T)a.invV;
-    }
-  }
-  cx<T>* base = a.spec + p * a.probStride + outer * a.outerStride + kx0;
-  const int w = min(TX, a.Pu - kx0);
-  for (int idx = threadIdx.x; idx < NIN * N * TX; idx += blockDim.x) {
-    const int col = idx % TX, j = (idx / TX) % N, c = idx / (TX * N);
-    const int line = (OP == OP_INV_SOL && c == 1) ? 2 : c;   // OP_INV_SOL: b goes to line 2
-    if (col < w)
-      cp_async<(int)sizeof(cx<T>)>(&sm[(line * TX + col) * C::LS + pad(j)],
-                                   &base[c * a.compStride + j * a.rowStride + col]);
-  }
-  cp_async_commit();
-  FillTw<T, N, 1, TW_MAX>::run(tw, a.twg);
-  cp_async_wait<0>();
-  __syncthreads();
-  if constexpr (OP == OP_INV || OP == OP_INV_SCALE || OP == OP_INV_SOL) {
-    if constexpr (OP == OP_INV_SOL) {
-      // line 1 = i d1(ky) b: the axis-1 derivative of chi before its inverse
-      // transform (the axis-2 one, a factor per column, is applied at the store)
-      for (int idx = threadIdx.x; idx < N * TX; idx += blockDim.x) {
-        const int col = idx % TX, j = idx / TX;
-        const cx<T> b = sm[(2 * TX + col) * C::LS + pad(j)];
-        sm[(1 * TX + col) * C::LS + pad(j)] = cscale(mul_i(b), a.sym.d1[j]);
-      }
-      __syncthreads();
-    }
-    if constexpr (OP == OP_INV_SCALE) {
-      const T s = (T)a.invV;
-      for (int idx = threadIdx.x; idx < NC * N * TX; idx += blockDim.x) {
-        const int col = idx % TX, j = (idx / TX) % N, c = idx / (TX * N);
-        cx<T>& x = sm[(c * TX + col) * C::LS + pad(j)];
-        x = cscale(x, s);
-      }
-      __syncthreads();
-    }
-    s_fft<T, N, OP, NC, TX, +1, NC * TX>(sm, tw, w);
-  } else {
-    s_fft<T, N, OP, NC, TX, -1, NIN * TX>(sm, tw, w);
-  }
-  if constexpr (OP == OP_FWD_SOL) {
-    // s'' = s' + i d1(ky) tau_1 into line 1
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < N * TX; idx += blockDim.x) {
-      const int col = idx % TX, j = idx / TX;
-      cx<T>& t1 = sm[(1 * TX + col) * C::LS + pad(j)];
-      t1 = sm[(2 * TX + col) * C::LS + pad(j)] + cscale(mul_i(t1), a.sym.d1[j]);
-    }
-  }
-  if constexpr (OP == OP_DERIV) {
-    __syncthreads();
-    const T invV = (T)a.invV;
-    for (int idx = threadIdx.x; idx < NC * N * TX; idx += blockDim.x) {
-      const int col = idx % TX, j = (idx / TX) % N, c = idx / (TX * N);
-      if (col >= w) continue;
-      const T d = a.dm == 0 ? a.sym.d0[j] : (a.dm == 1 ? a.sym.d1[outer] : a.sym.d2[kx0 + col]);
-      cx<T>& x = sm[(c * TX + col) * C::LS + pad(j)];
-      x = cscale(mul_i(x), d * invV);
-    }
-    __syncthreads();
-    s_fft<T, N, OP, NC, TX, +1, NC * TX>(sm, tw, w);
-  }
-  if constexpr (OP == OP_STOKES || OP == OP_SOLUTE) {
-    __syncthreads();
-    const T invV = opar[4];
-    const int ky = outer;
-    const T d1 = a.sym.d1[ky], l1 = a.sym.l1[ky];
-    T acc0 = 0, acc1 = 0, acc2 = 0;
-    // hoisted parameters of the operator
-    T nu = 0, beta = 0, b = 0, A0 = 0, B00 = 0, B01 = 0, B02 = 0;
-    if constexpr (OP == OP_STOKES) {
-      nu = opar[0];
-      beta = opar[1];
-      b = opar[2];
-    } else {
-      A0 = opar[0];
-      B00 = opar[1];
-      B01 = opar[2];
-      B02 = opar[3];
-    }
-    // The operator state (q^ and div^, or chi^) is read and rewritten in place:
-    // each chunk loads its state before any store (see k_x_stokes_local).
-    // The block size is a multiple of TX, so a thread keeps one tile column and
-    // its kx symbols and Parseval weight stay in registers.
-    static_assert(C::NT % TX == 0, "one column per thread");
-    constexpr int TOT = N * TX, CH = 4;
-    const int col = threadIdx.x % TX, kx = kx0 + col;
-    const bool colok = col < w;
-    const T d2 = colok ? a.sym.d2[kx] : (T)0, l2 = colok ? a.sym.l2[kx] : (T)0;
-    const T wgt = (kx == 0 || kx == a.nkx) ? (T)1 : (T)2;
-    const T l12 = l1 + l2, d12 = d1 * d1 + d2 * d2;
-    const long long gcol = (long long)p * a.compStride + (long long)outer * a.outerStride + kx0 + col;
-#pragma unroll 1
-    for (int base = 0; base < TOT; base += CH * C::NT) {
-      bool ok[CH];
-      long long gis[CH];
-      cx<T> sa[CH], sb[CH];
-#pragma unroll
-      for (int k = 0; k < CH; ++k) {
-        const int idx = base + k * C::NT + threadIdx.x;
-        const int j = idx / TX;
-        ok[k] = idx < TOT && colok;
-        gis[k] = gcol + (long long)j * a.rowStride;
-        sa[k] = ok[k] ? a.st0[gis[k]] : mk<T>(0, 0);
-        if constexpr (OP == OP_STOKES) sb[k] = ok[k] ? a.st1[gis[k]] : mk<T>(0, 0);
-      }
-#pragma unroll
-      for (int k = 0; k < CH; ++k) {
-        if (!ok[k]) continue;
-        const int idx = base + k * C::NT + threadIdx.x;
-        const int j = idx / TX;
-        const long long gi = gis[k];
-        const T d0 = a.sym.d0[j], l0 = a.sym.l0[j];
-        const T L = l0 + l12, dd = d0 * d0 + d12;
-        const bool k0 = (j == 0 && ky == 0 && kx == 0);
-        cx<T>* s0 = &sm[(0 * TX + col) * C::LS + pad(j)];
-        cx<T>* s1 = &sm[(1 * TX + col) * C::LS + pad(j)];
-        if constexpr (OP == OP_STOKES) {
-          cx<T>* s2 = &sm[(2 * TX + col) * C::LS + pad(j)];
-          const cx<T> qh = sa[k];
-          const cx<T> dprev = sb[k];
-          // r = w^ - i d q^ (+ g V at k = 0)
-          const cx<T> iq = mul_i(qh);
-          cx<T> r0 = *s0 - cscale(iq, d0), r1 = *s1 - cscale(iq, d1), r2 = *s2 - cscale(iq, d2);
-          if (k0) {
-            const StokesDev& P = a.sprm[p];
-            const T Vt = (T)(1.0 / a.invV);
-            r0.x += (T)P.g[0] * Vt;
-            r1.x += (T)P.g[1] * Vt;
-            r2.x += (T)P.g[2] * Vt;
-          }
-          // Eq. 13: (nu L + b) u^ + beta d (d.u^) = r, solved as
-          //   d.u^ = d.r / (c + beta |d|^2),  u^ = (r - beta d (d.u^)) / c,  c = nu L + b
-          const T c0 = nu * L + b;
-          const T ic0 = (T)1 / c0;
-          const cx<T> dr = cscale(r0, d0) + cscale(r1, d1) + cscale(r2, d2);
-          const cx<T> du = cscale(dr, (T)1 / (c0 + beta * dd));
-          const cx<T> f = cscale(du, beta);
-          const cx<T> u0 = cscale(r0 - cscale(f, d0), ic0);
-          const cx<T> u1 = cscale(r1 - cscale(f, d1), ic0);
-          const cx<T> u2 = cscale(r2 - cscale(f, d2), ic0);
-          // div u^ = i d.u^ (taken from the solve, free of the cancellation of
-          // summing d_c u^_c when beta is large); Eq. 9: q^ <- q^ - beta div u^
-          const cx<T> dv = mul_i(du);
-          const cx<T> qn = qh - cscale(dv, beta);
-          a.st0[gi] = qn;
-          a.st1[gi] = dv;
-          const cx<T> ddv = dv - dprev;
-          acc0 += wgt * cabs2(dv);
-          acc1 += wgt * cabs2(ddv);
-          acc2 += wgt * cabs2(qn);
-          if (k0) {
-            a.sprm[p].mean_u[0] = (double)u0.x * a.invV;
-            a.sprm[p].mean_u[1] = (double)u1.x * a.invV;
-            a.sprm[p].mean_u[2] = (double)u2.x * a.invV;
-          }
-          *s0 = cscale(u0, invV);
-          *s1 = cscale(u1, invV);
-          *s2 = cscale(u2, invV);
-        } else {
-          // F^ = s^ + i d.tau^ (Eq. 18 in Fourier space): the axis-2 and axis-1
-          // terms were added in the x and y passes, line 1 holds s''
-          const cx<T> F = *s1 + mul_i(cscale(*s0, d0));
-          // Eq. 20: chi^ = F^ / (i B0.d + A0 L), chi^(0) = 0
-          const T dre = A0 * L, dim = B00 * d0 + B01 * d1 + B02 * d2;
-          cx<T> chi = mk<T>(0, 0);
-          if (!k0) {
-            const T den = (T)1 / (dre * dre + dim * dim);
-            chi = mk<T>((F.x * dre + F.y * dim) * den, (F.y * dre - F.x * dim) * den);
-          }
-          const cx<T> dch = chi - sa[k];
-          a.st0[gi] = chi;
-          acc0 += wgt * cabs2(dch);
-          acc1 += wgt * dd * cabs2(dch);
-          // i d0 chi^ and chi^, normalised for the inverse transform (the
-          // axis-1 and axis-2 derivatives are taken in the later passes)
-          const cx<T> cs = cscale(chi, invV);
-          *s0 = cscale(mul_i(cs), d0);
-          *s1 = cs;
-        }
-      }
-    }
-    T v3[3] = {acc0, acc1, acc2};
-    const int nb = gridDim.x * gridDim.y;
-    block_sum_store<3>(v3, red, a.part + ((long long)p * nb + blockIdx.y * gridDim.x + blockIdx.x) * 4);
-    __syncthreads();
-    s_fft<T, N, OP, NC, TX, +1, NOUT * TX>(sm, tw, w);
-  }
-  __syncthreads();
-  // OP_INV_SOL: line 2 leaves as i d2(kx) b; with NT a multiple of TX every
-  // thread stores one column, whose symbol is read once
-  constexpr bool fixed_col = C::NT % TX == 0;
-  T d2c = (T)0;
-  if constexpr (OP == OP_INV_SOL && fixed_col)
-    if ((int)threadIdx.x % TX < w) d2c = a.sym.d2[kx0 + (int)threadIdx.x % TX];
-  for (int idx = threadIdx.x; idx < NOUT * N * TX; idx += blockDim.x) {
-    const int col = idx % TX, j = (idx / TX) % N, c = idx / (TX * N);
-    if (col < w) {
-      cx<T> x = sm[(c * TX + col) * C::LS + pad(j)];
-      if constexpr (OP == OP_INV_SOL)
-        if (c == 2) x = cscale(mul_i(x), fixed_col ? d2c : a.sym.d2[kx0 + col]);
-      base[c * a.compStride + j * a.rowStride + col] = x;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
 // FP64 reductions over real fields
 // ---------------------------------------------------------------------------
 // sums[p][0..2] = sum u_c ; [3..5] = sum over pore u_c ; [6] = pore voxels.
@@ -1195,5 +904,3 @@ __global__ void k_q_from_a(const cx<T>* __restrict__ ah, cx<T>* __restrict__ q, 
 }
 
 }  // namespace acm
-
-#include "acm_rpass.cuh"

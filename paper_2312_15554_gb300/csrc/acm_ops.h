@@ -18,8 +18,8 @@ struct Ops {
   // blocks per problem of the x-passes and of a z-pass (number of partial sums)
   static int x_blocks(const Geo& g);
   static int z_blocks(const Geo& g, int op);
-  // tile width (columns) a strided pass launches with under g's tile choice, and
-  // whether the choice `shift` (-1, 0, +1) has its own compiled variant
+  // tile width (columns) a strided pass reports under g's tile choice, and
+  // whether the choice `shift` (-1 .. 4) is one of its own
   static int pass_tx(const Geo& g, int axis, int op, int nc);
   static bool tx_variant(int n, int op, int nc, int shift);
 

@@ -8,9 +8,8 @@
 
 namespace acm {
 
-// Tile width (kx columns) of a strided pass: about 256 threads per block (many
-// resident blocks hide the memory latency better than wide tiles), at least 2
-// columns, and at most 64 KB of shared memory.
+// The default tile width (kx columns) a strided pass reports: about 256 threads
+// over its components, at least 2 columns, at most 64 KB of shared memory.
 constexpr int pick_tx(int csize, int N, int NC) {
   int tl = N / ept(N);
   int tx = 16;
@@ -150,11 +149,11 @@ static cudaError_t l_x_c2r(const Geo& g, int nprob, int nc, const void* spec, lo
   return cudaErrorInvalidValue;
 }
 
-// Autotuner candidates: the passes of the solver loops at N >= 64 also exist
-// with half, double and four times the default tile width, when the variant
-// stays within 2..32 columns, 1536 line threads (run in rounds of at most 512
-// or 1024) and 200 KB of shared memory. Wide tiles read longer row segments,
-// which matters most along the slowest axis.
+// Tile choices of a pass (Geo::txs): 0 lets the pass pick its width from the
+// grid; the solver passes at N >= 64 also take -1, 1, 2 (half, double, four
+// times the default width reported, where that number stays within 2..32 columns,
+// 1536 line threads and 200 KB) and, at N = 64, 128 and 256, 3 and 4 (a full and
+// a half 128-byte row segment, reported as -W).
 template <int N, int OP, int NC>
 constexpr bool tunable() {
   return N >= 64 && ((OP == OP_FWD && NC == 3) || (OP == OP_INV && NC == 3) || OP == OP_STOKES || OP == OP_SOLUTE ||
@@ -167,16 +166,16 @@ constexpr bool tx_ok() {
          (NC * TX * line_stride(N, N / ept(N), TX, wave_slots<T>()) + tw_total(N)) * (int)sizeof(cx<T>) <= 200 * 1024;
 }
 
-// The register-resident variant (acm_rpass.cuh) of a tunable pass: lines of
-// 64, 128 or 256 points.
 template <typename T, int N, int OP, int NC>
 constexpr bool rr_ok() {
   return (N == 64 || N == 128 || N == 256) && tunable<N, OP, NC>();
 }
 
-// tile width of (T, N, OP, NC) under the choice `shift`; the register-resident
-// variants (shift 3: W = rr_wdef, shift 4: W = rr_wdef / 2 columns per block)
-// report -W
+// columns of one 128-byte row segment (16 in FP32, 8 in FP64)
+template <typename T>
+constexpr int rr_wdef() { return 128 / (int)sizeof(cx<T>); }
+
+// the width (T, N, OP, NC) reports under the choice `shift`
 template <typename T, int N, int OP, int NC>
 constexpr int resolved_tx(int shift) {
   constexpr int TX0 = pick_tx((int)sizeof(cx<T>), N, NC);
@@ -190,6 +189,42 @@ constexpr int resolved_tx(int shift) {
     if (shift == 2 && tx_ok<T, N, OP, NC, TX0 * 4>()) return TX0 * 4;
   }
   return TX0;
+}
+
+// Compiled widths of (T, N): powers of two from max(4, the width that fills a
+// warp) to a full 128-byte row segment (half of one at N = 512, where three
+// groups of wider tiles pass 1024 threads), or the one that fills a warp alone.
+template <typename T, int N>
+constexpr int lp_wmin() {
+  constexpr int TL = N / lp_ept<T>(N);
+  return TL >= 8 ? 4 : 32 / TL;
+}
+template <typename T, int N>
+constexpr int lp_wmax() {
+  constexpr int m = N == 512 ? rr_wdef<T>() / 2 : rr_wdef<T>();
+  return m < lp_wmin<T, N>() ? lp_wmin<T, N>() : m;
+}
+
+// The width a pass runs with. Asked for one, the nearest compiled. Left to
+// itself, the widest that gives a problem two tiles per SM (152), at most half
+// a row segment in the z operators (their three groups of a full segment fill an
+// SM's thread budget with one block), so that small grids spread over the SMs and
+// large ones read long segments. Depends on the grid alone: a problem's partial
+// sums do not depend on how many share its launch.
+template <typename T, int N>
+static int lp_width(const Geo& g, int axis, int op, int reported) {
+  constexpr int lo = lp_wmin<T, N>(), hi = lp_wmax<T, N>();
+  const int sh = g.txs[sizeof(T) == 8][axis][op];
+  int w = hi;
+  if (sh == 0) {
+    if ((op == OP_STOKES || op == OP_SOLUTE) && w > lo) w /= 2;
+    const int nouter = axis == 1 ? g.n0 : g.n1;
+    while (w > lo && rr_tiles(g.Pu, nouter, w).nlive < 304) w /= 2;
+    return w;
+  }
+  const int want = reported < 0 ? -reported : reported;
+  while (w > lo && w > want) w /= 2;
+  return w;
 }
 
 template <typename T>
@@ -208,7 +243,6 @@ static PassArgs<T> pass_args(const Geo& g, int axis, void* spec, long long probS
     a.outerStride = g.P;
   }
   a.Pu = g.Pu;
-  a.n1 = g.n1;
   a.sym = sym;
   a.twg = (const cx<T>*)tw;
   a.st0 = (cx<T>*)st0;
@@ -223,69 +257,45 @@ static PassArgs<T> pass_args(const Geo& g, int axis, void* spec, long long probS
   return a;
 }
 
-template <typename T, int N, int OP, int NC, int TX>
-static cudaError_t l_pass_kt(const Geo& g, int axis, int nprob, void* spec, long long probStride, const Sym<T>& sym,
-                             const void* tw, void* st0, void* st1, StokesDev* sprm, SoluteDev* cprm, double* part,
-                             cudaStream_t s, int dm) {
-  using C = SCfg<T, N, OP, NC, TX>;
-  static const cudaError_t attr = set_smem(k_strided<T, N, OP, NC, TX>, C::SMEM);
+template <typename T, int N, int OP, int W, bool SEG>
+static cudaError_t l_pass_w(const PassArgs<T>& a, int nc, int nprob, cudaStream_t s) {
+  using C = LCfg<T, N, W>;
+  constexpr int smem = lp_smem<T, N, OP, W>(), threads = lp_groups(OP) * C::NT;
+  constexpr auto k = [] {
+    if constexpr (OP == OP_STOKES || OP == OP_SOLUTE) return k_lpass_z<T, N, OP, W, SEG>;
+    else if constexpr (OP == OP_FWD_SOL) return k_lpass_fsol<T, N, OP, W, SEG>;
+    else if constexpr (OP == OP_INV_SOL) return k_lpass_isol<T, N, OP, W, SEG>;
+    else return k_lpass<T, N, OP, W, SEG>;
+  }();
+  static const cudaError_t attr = set_smem(k, smem);
   if (attr != cudaSuccess) return attr;
-  const PassArgs<T> a = pass_args<T>(g, axis, spec, probStride, sym, tw, st0, st1, sprm, cprm, part, dm);
-  const int nouter = axis == 1 ? g.n0 : g.n1;
-  dim3 grid((g.Pu + TX - 1) / TX, nouter, nprob);
-  k_strided<T, N, OP, NC, TX><<<grid, C::NT, C::SMEM, s>>>(a);
+  const int nlive = rr_tiles(a.Pu, a.nouter, W).nlive;
+  const dim3 grid = OP == OP_FWD_SOL     ? dim3((nlive + 1) / 2 * 3, nprob)
+                    : OP == OP_INV_SOL   ? dim3(3 * nlive, nprob)
+                    : lp_groups(OP) == 1 ? dim3(nlive, nc, nprob)
+                                         : dim3(nlive, nprob);
+  k<<<grid, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename T, int N, int OP, int NC, int W>
-static cudaError_t l_pass_rr(const Geo& g, int axis, int nprob, void* spec, long long probStride, const Sym<T>& sym,
-                             const void* tw, void* st0, void* st1, StokesDev* sprm, SoluteDev* cprm, double* part,
-                             cudaStream_t s) {
-  using C = RCfg<T, N, W>;
-  constexpr int smem = rr_smem<T, N, OP, NC, W>();
-  constexpr bool wide = rr_y_wide<T, OP, W>() && N == 256;
-  static const cudaError_t attr = [] {
-    if constexpr (wide) return set_smem(k_rstrided_w<T, N, OP, NC, W>, smem);
-    else return set_smem(k_rstrided<T, N, OP, NC, W>, smem);
-  }();
-  if (attr != cudaSuccess) return attr;
-  const PassArgs<T> a = pass_args<T>(g, axis, spec, probStride, sym, tw, st0, st1, sprm, cprm, part, 0);
-  const RTiles tl = rr_tiles(g.Pu, a.nouter, W);
-  if constexpr (wide) k_rstrided_w<T, N, OP, NC, W><<<nprob * tl.nlive, C::NT, smem, s>>>(a);
-  else k_rstrided<T, N, OP, NC, W><<<nprob * tl.nlive, C::NT, smem, s>>>(a);
-  return cudaGetLastError();
+template <typename T, int N, int OP, int W, bool SEG>
+static cudaError_t l_pass_pick(int w, const PassArgs<T>& a, int nc, int nprob, cudaStream_t s) {
+  if constexpr (W > lp_wmin<T, N>())
+    if (w < W) return l_pass_pick<T, N, OP, W / 2, SEG>(w, a, nc, nprob, s);
+  return l_pass_w<T, N, OP, W, SEG>(a, nc, nprob, s);
 }
 
 template <typename T, int N, int OP, int NC>
 static cudaError_t l_pass_k(const Geo& g, int axis, int nprob, void* spec, long long probStride, const Sym<T>& sym,
                             const void* tw, void* st0, void* st1, StokesDev* sprm, SoluteDev* cprm, double* part,
                             cudaStream_t s, int dm) {
-  constexpr int TX0 = pick_tx((int)sizeof(cx<T>), N, NC);
-  if constexpr (rr_ok<T, N, OP, NC>()) {
-    const int sh = g.txs[sizeof(T) == 8][axis][OP];
-    if (sh == 3)
-      return l_pass_rr<T, N, OP, NC, rr_wdef<T>()>(g, axis, nprob, spec, probStride, sym, tw, st0, st1, sprm, cprm,
-                                                   part, s);
-    if (sh == 4)
-      return l_pass_rr<T, N, OP, NC, rr_wdef<T>() / 2>(g, axis, nprob, spec, probStride, sym, tw, st0, st1, sprm,
-                                                       cprm, part, s);
-  }
-  if constexpr (tunable<N, OP, NC>()) {
-    const int sh = g.txs[sizeof(T) == 8][axis][OP];
-    if constexpr (tx_ok<T, N, OP, NC, TX0 / 2>())
-      if (sh < 0)
-        return l_pass_kt<T, N, OP, NC, TX0 / 2>(g, axis, nprob, spec, probStride, sym, tw, st0, st1, sprm, cprm,
-                                                part, s, dm);
-    if constexpr (tx_ok<T, N, OP, NC, TX0 * 2>())
-      if (sh == 1)
-        return l_pass_kt<T, N, OP, NC, TX0 * 2>(g, axis, nprob, spec, probStride, sym, tw, st0, st1, sprm, cprm,
-                                                part, s, dm);
-    if constexpr (tx_ok<T, N, OP, NC, TX0 * 4>())
-      if (sh == 2)
-        return l_pass_kt<T, N, OP, NC, TX0 * 4>(g, axis, nprob, spec, probStride, sym, tw, st0, st1, sprm, cprm,
-                                                part, s, dm);
-  }
-  return l_pass_kt<T, N, OP, NC, TX0>(g, axis, nprob, spec, probStride, sym, tw, st0, st1, sprm, cprm, part, s, dm);
+  const PassArgs<T> a = pass_args<T>(g, axis, spec, probStride, sym, tw, st0, st1, sprm, cprm, part, dm);
+  const int sh = g.txs[sizeof(T) == 8][axis][OP];
+  const int w = lp_width<T, N>(g, axis, OP, resolved_tx<T, N, OP, NC>(sh));
+  // the tuned row-segment widths keep their own rounding (lp_ifft_dit, cmul_fma)
+  if constexpr (rr_ok<T, N, OP, NC>() && sizeof(T) == 4)
+    if (sh >= 3) return l_pass_pick<T, N, OP, lp_wmax<T, N>(), true>(w, a, NC, nprob, s);
+  return l_pass_pick<T, N, OP, lp_wmax<T, N>(), false>(w, a, NC, nprob, s);
 }
 
 template <typename T, int N>
@@ -294,7 +304,6 @@ static int l_pass_tx(int op, int nc, int shift) {
   if (op == OPV && nc == NCV) return resolved_tx<T, N, OPV, NCV>(shift);
   ACM_TX(OP_FWD, 1)
   ACM_TX(OP_FWD, 3)
-  ACM_TX(OP_FWD, 4)
   ACM_TX(OP_INV, 1)
   ACM_TX(OP_INV, 3)
   ACM_TX(OP_INV_SCALE, 1)
@@ -307,6 +316,12 @@ static int l_pass_tx(int op, int nc, int shift) {
   return 0;
 }
 
+// the width a pass runs with under g's choice
+template <typename T, int N>
+static int l_pass_w(const Geo& g, int axis, int op, int nc) {
+  return lp_width<T, N>(g, axis, op, l_pass_tx<T, N>(op, nc, g.txs[sizeof(T) == 8][axis][op]));
+}
+
 template <typename T, int N>
 static cudaError_t l_pass(const Geo& g, int axis, int op, int nc, int nprob, void* spec, long long ps,
                           const Sym<T>& sym, const void* tw, void* st0, void* st1, StokesDev* sprm, SoluteDev* cprm,
@@ -316,7 +331,6 @@ static cudaError_t l_pass(const Geo& g, int axis, int op, int nc, int nprob, voi
     return l_pass_k<T, N, OPV, NCV>(g, axis, nprob, spec, ps, sym, tw, st0, st1, sprm, cprm, part, s, dm);
   ACM_PASS(OP_FWD, 1)
   ACM_PASS(OP_FWD, 3)
-  ACM_PASS(OP_FWD, 4)
   ACM_PASS(OP_INV, 1)
   ACM_PASS(OP_INV, 3)
   ACM_PASS(OP_INV_SCALE, 1)
@@ -368,9 +382,20 @@ bool Ops<T>::tx_variant(int n, int op, int nc, int shift) {
 template <typename T>
 int Ops<T>::z_blocks(const Geo& g, int op) {
   const int nc = op == P_SOLUTE ? 2 : 3;
-  const int tx = pass_tx(g, 0, op, nc);
-  if (tx < 0) return rr_tiles(g.Pu, g.n1, -tx).nlive;   // register-resident: one record per live tile
-  return ((g.Pu + tx - 1) / tx) * g.n1;
+  auto width = [&]() -> int {
+    switch (g.n0) {
+      case 1: return l_pass_w<T, 1>(g, 0, op, nc);
+      case 8: return l_pass_w<T, 8>(g, 0, op, nc);
+      case 16: return l_pass_w<T, 16>(g, 0, op, nc);
+      case 32: return l_pass_w<T, 32>(g, 0, op, nc);
+      case 64: return l_pass_w<T, 64>(g, 0, op, nc);
+      case 128: return l_pass_w<T, 128>(g, 0, op, nc);
+      case 256: return l_pass_w<T, 256>(g, 0, op, nc);
+      case 512: return l_pass_w<T, 512>(g, 0, op, nc);
+      default: return 1;
+    }
+  };
+  return rr_tiles(g.Pu, g.n1, width()).nlive;
 }
 
 template <typename T>

@@ -64,7 +64,8 @@ struct Geo {
   long long us; // stride of the advecting velocity between problems (0: shared)
   int lph;      // problems per indicator: problem p uses H + (p / lph) * hs
   // tile-width choice of the strided passes per [precision (FP64 = 1)][axis][pass op]:
-  // -1 half, 0 default, +1 double, +2 four times the default width (set by the autotuner)
+  // 0 by the grid; -1 half, +1 double, +2 four times the default width; +3, +4 row
+  // segments of 128 and 64 bytes (set by the autotuner)
   signed char txs[2][2][8] = {};
 };
 

@@ -8,22 +8,65 @@ namespace acm {
 // ---------------------------------------------------------------------------
 // finalize kernels: deterministic FP64 sums of the partials, Eq. 10-12, Eq. 22
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void sum_partials(const double* __restrict__ part, int nblk, int stride, int nval,
-                                             double* out, double* red) {
-  double acc[5] = {0, 0, 0, 0, 0};
-  for (int i = threadIdx.x; i < nblk; i += blockDim.x)
-    for (int k = 0; k < nval; ++k) acc[k] += part[(long long)i * stride + k];
-  block_sum_store<5>(acc, red, out);
+// One finalize block per problem. FP64 runs on two lanes an SM, so the block sums
+// eight values at once by halving: a warp's lanes exchange half of their values at
+// each of the first three steps (4 + 2 + 1 + 1 + 1 additions a lane, against 40
+// for eight butterflies), and the residuals, tolerances and penalties are formed
+// by one lane each. A problem's whole step took 18 us a launch as eight butterflies
+// and one thread's chain of square roots, divisions and loads of its control block.
+constexpr int FIN_VALS = 8;
+constexpr int FIN_MAXW = 32;
+
+// Sums v[0..7] over the block; lane k (mod 8) of warp 0 returns the total of value
+// k. scratch: FIN_VALS * FIN_MAXW doubles. Deterministic for a fixed block size.
+__device__ __forceinline__ double block_sum8(double (&v)[FIN_VALS], double* scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  // after the step over bit `o` a lane holds the values whose index has the lane's
+  // bit there: value index k = lane & 7
+#pragma unroll
+  for (int o = 4, n = 4; o >= 1; o >>= 1, n >>= 1) {
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      const bool up = lane & o;
+      const double keep = up ? v[i + n] : v[i], give = up ? v[i] : v[i + n];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  double a = v[0];
+  a += __shfl_xor_sync(0xffffffffu, a, 8);
+  a += __shfl_xor_sync(0xffffffffu, a, 16);
+  if (lane < FIN_VALS) scratch[warp * FIN_VALS + lane] = a;
   __syncthreads();
+  double r = 0.0;
+  if (warp == 0) {
+    for (int w = lane >> 3; w < nw; w += 4) r += scratch[w * FIN_VALS + (lane & 7)];
+    r += __shfl_xor_sync(0xffffffffu, r, 8);
+    r += __shfl_xor_sync(0xffffffffu, r, 16);
+  }
+  return r;
+}
+
+// adds the records part[i][0..NV) (stride doubles apart, pairs 16-byte aligned) of
+// the thread's share to v[0..NV)
+template <int NV>
+__device__ __forceinline__ void add_partials(const double* __restrict__ part, int nblk, int stride, double* v) {
+#pragma unroll 4
+  for (int i = threadIdx.x; i < nblk; i += blockDim.x) {
+    const double2* q = reinterpret_cast<const double2*>(part + (long long)i * stride);
+#pragma unroll
+    for (int k = 0; k < NV; k += 2) {
+      const double2 x = q[k / 2];
+      v[k] += x.x;
+      if (k + 1 < NV) v[k + 1] += x.y;
+    }
+  }
 }
 
 // Stagnation test of an FP32 phase (off when win = 0): the distance to the
 // tolerance m = max_k r[k] / t[k] must fall below STALL_DROP times its best
 // value within `win` iterations, else the phase has reached its rounding floor.
-__device__ __forceinline__ bool stalled(int win, int& n, double& best, const double* r, const double* t, int k) {
+__device__ __forceinline__ bool stalled(int win, int& n, double& best, double m) {
   if (win <= 0) return false;
-  double m = 0.0;
-  for (int i = 0; i < k; ++i) m = fmax(m, t[i] > 0.0 ? r[i] / t[i] : r[i]);
   if (m < STALL_DROP * best) {
     best = m;
     n = 0;
@@ -32,65 +75,90 @@ __device__ __forceinline__ bool stalled(int win, int& n, double& best, const dou
   return ++n >= win;
 }
 
-__global__ void __launch_bounds__(256) k_stokes_finalize(StokesDev* __restrict__ prm, const double* __restrict__ part_x,
-                                                        int nbx, const double* __restrict__ part_z, int nbz,
-                                                        double V, double* __restrict__ hist, int hist_cap) {
-  __shared__ double red[5 * 32];
-  __shared__ double sx[5], sz[5];
+__device__ __forceinline__ double shfl(double x, int src) { return __shfl_sync(0xffffffffu, x, src); }
+
+__global__ void __launch_bounds__(1024) k_stokes_finalize(StokesDev* __restrict__ prm, const double* __restrict__ part_x,
+                                                         int nbx, const double* __restrict__ part_z, int nbz,
+                                                         double V, double* __restrict__ hist, int hist_cap) {
+  __shared__ double red[FIN_VALS * FIN_MAXW];
   const int p = blockIdx.x;
   StokesDev* P = prm + p;
   if (P->done) return;
-  sum_partials(part_x + (long long)p * nbx * 8, nbx, 8, 5, sx, red);
-  sum_partials(part_z + (long long)p * nbz * 4, nbz, 4, 3, sz, red);
-  if (threadIdx.x != 0) return;
-  const double alpha = P->psi[0], beta = P->psi[1], b = P->psi[2];
-  double r[6];
-  r[0] = sqrt(sx[0]);
-  r[1] = alpha * sqrt(sx[1]);
-  r[2] = sqrt(sz[0] / V);
-  r[3] = beta * sqrt(sz[1] / V);
-  r[4] = sqrt(sx[2]);
-  r[5] = b * sqrt(sx[3]);
-  const double nl = sqrt(sx[4]), nq = sqrt(sz[2] / V), na = nl;  // a = H lambda
-  const double e = P->eps, s13 = sqrt(3.0 * V) * e, s2 = sqrt(V) * e;
-  double t[6];
-  t[0] = s13 + e * fmax(r[0], nl);
-  t[1] = s13 + e * nl;
-  t[2] = s2 + e * fmax(r[2], nq);
-  t[3] = s2 + e * nq;
-  t[4] = s13 + e * fmax(r[4], na);
-  t[5] = s13 + e * na;
-  bool conv = true, finite = true;
-  for (int k = 0; k < 6; ++k) {
-    P->res[k] = r[k];
-    P->tol[k] = t[k];
-    conv = conv && (r[k] <= t[k]);
-    finite = finite && isfinite(r[k]);
+  const int lane = threadIdx.x;
+  const bool first = threadIdx.x < 32;
+  // warp 0 reads the control block while the partial sums travel: lane k holds
+  // entry k of the vectors
+  const int k3 = lane < 3 ? lane : 0;
+  double psi = 0, phi = 0, tau = 0, psi_min = 0, mean = 0, e = 0;
+  int adaptive = 0, max_iter = 0, iter = 0, iter_base = 0, stall_win = 0;
+  if (first) {
+    psi = P->psi[k3];
+    phi = P->phi[k3];
+    tau = P->tau[k3];
+    psi_min = P->psi_min[k3];
+    mean = P->mean_u[k3];
+    e = P->eps;
+    adaptive = P->adaptive;
+    max_iter = P->max_iter;
+    iter = P->iter;
+    iter_base = P->iter_base;
+    stall_win = P->stall_win;
   }
-  P->iter += 1;
-  const int it = P->iter;
-  if (hist && it + P->iter_base <= hist_cap) {
-    double* h = hist + ((long long)p * hist_cap + (it + P->iter_base - 1)) * STOKES_HIST;
-    for (int k = 0; k < 6; ++k) h[k] = r[k];
-    for (int k = 0; k < 6; ++k) h[6 + k] = t[k];
-    h[12] = alpha;
-    h[13] = beta;
-    h[14] = b;
-    for (int k = 0; k < 3; ++k) h[15 + k] = P->mean_u[k];
-    h[18] = 0.0;
-    h[19] = 0.0;
+  // values 0..4: the x pass (||Hu~||^2, ||H(u~ - u~_old)||^2, ||u - u~||^2,
+  // ||u - u_old||^2, ||lambda||^2), 5..7: the z pass (V times ||div u||^2,
+  // ||div (u - u_old)||^2, ||q||^2)
+  double v[FIN_VALS] = {0, 0, 0, 0, 0, 0, 0, 0};
+  add_partials<5>(part_x + (long long)p * nbx * 8, nbx, 8, v);
+  add_partials<3>(part_z + (long long)p * nbz * 4, nbz, 4, v + 5);
+  const double total = block_sum8(v, red);
+  if (!first) return;
+  // lane k: the norm of value k (all 32 lanes compute, eight distinct values)
+  const double nrm = sqrt((lane & 7) >= 5 ? total / V : total);
+  const double n0 = shfl(nrm, 0), n1 = shfl(nrm, 1), n2 = shfl(nrm, 2), n3 = shfl(nrm, 3), nl = shfl(nrm, 4);
+  const double z0 = shfl(nrm, 5), z1 = shfl(nrm, 6), nq = shfl(nrm, 7);
+  const double alpha = shfl(psi, 0), beta = shfl(psi, 1), b = shfl(psi, 2);
+  // lane k < 6: residual k (Eq. 10) and its tolerance (Eq. 11-12); a = H lambda
+  const double r = lane == 0 ? n0 : lane == 1 ? alpha * n1 : lane == 2 ? z0 : lane == 3 ? beta * z1
+                   : lane == 4 ? n2 : b * n3;
+  const bool pair2 = (lane >> 1) == 1;
+  const double s = sqrt(pair2 ? V : 3.0 * V) * e, nm = pair2 ? nq : nl;
+  const double t = s + e * ((lane & 1) ? nm : fmax(r, nm));
+  const unsigned six = 0x3fu;
+  const bool conv = (__ballot_sync(0xffffffffu, r <= t) & six) == six;
+  const bool finite = (__ballot_sync(0xffffffffu, isfinite(r)) & six) == six;
+  const int it = iter + 1;
+  if (lane < 6) {
+    P->res[lane] = r;
+    P->tol[lane] = t;
   }
-  for (int k = 0; k < 3; ++k) {
-    P->psi_last[k] = P->psi[k];
-    P->psi_prev[k] = P->psi[k];
+  if (hist && it + iter_base <= hist_cap) {
+    double* h = hist + ((long long)p * hist_cap + (it + iter_base - 1)) * STOKES_HIST;
+    if (lane < 6) {
+      h[lane] = r;
+      h[6 + lane] = t;
+    }
+    if (lane < 3) {
+      h[12 + lane] = psi;
+      h[15 + lane] = mean;
+    }
+    if (lane < 2) h[18 + lane] = 0.0;
   }
-  if (P->adaptive) {
-    for (int k = 0; k < 3; ++k) {  // Eq. 22: pair k drives (alpha, beta, b)[k]
-      const double rp = r[2 * k], rd = r[2 * k + 1];
-      if (rp > P->tau[k] * rd) P->psi[k] = P->phi[k] * P->psi[k];
-      else if (rd > P->tau[k] * rp) P->psi[k] = fmax(P->psi[k] / P->phi[k], P->psi_min[k]);
+  const double rp = shfl(r, 2 * k3), rd = shfl(r, 2 * k3 + 1);
+  if (lane < 3) {
+    P->psi_last[lane] = psi;
+    P->psi_prev[lane] = psi;
+    if (adaptive) {  // Eq. 22: pair k drives (alpha, beta, b)[k]
+      if (rp > tau * rd) P->psi[lane] = phi * psi;
+      else if (rd > tau * rp) P->psi[lane] = fmax(psi / phi, psi_min);
     }
   }
+  double m = 0.0;
+  if (stall_win > 0) {
+    const double q = lane < 6 ? (t > 0.0 ? r / t : r) : 0.0;
+    for (int i = 0; i < 6; ++i) m = fmax(m, shfl(q, i));
+  }
+  if (lane != 0) return;
+  P->iter = it;
   if (!finite) {
     P->done = 1;
     P->status = ST_NONFINITE;
@@ -98,64 +166,78 @@ __global__ void __launch_bounds__(256) k_stokes_finalize(StokesDev* __restrict__
     P->done = 1;
     P->converged = 1;
     P->status = ST_OK;
-  } else if (stalled(P->stall_win, P->stall_n, P->stall_best, r, t, 6)) {
+  } else if (stalled(stall_win, P->stall_n, P->stall_best, m)) {
     P->done = 1;
     P->status = ST_STALLED;
-  } else if (it >= P->max_iter) {
+  } else if (it >= max_iter) {
     P->done = 1;
     P->status = ST_MAXITER;
   }
 }
 
-__global__ void __launch_bounds__(256) k_solute_finalize(SoluteDev* __restrict__ prm, const double* __restrict__ part_z,
-                                                        int nbz, double V, double* __restrict__ hist, int hist_cap) {
-  __shared__ double red[5 * 32];
-  __shared__ double sz[5];
+__global__ void __launch_bounds__(1024) k_solute_finalize(SoluteDev* __restrict__ prm, const double* __restrict__ part_z,
+                                                         int nbz, double V, double* __restrict__ hist, int hist_cap) {
+  __shared__ double red[FIN_VALS * FIN_MAXW];
   const int p = blockIdx.x;
   SoluteDev* P = prm + p;
   if (P->done) return;
-  sum_partials(part_z + (long long)p * nbz * 4, nbz, 4, 2, sz, red);
-  if (threadIdx.x != 0) return;
-  const double r1 = sqrt(sz[0] / V), r2 = sqrt(sz[1] / V);
-  const double t1 = sqrt(V) * P->eps, t2 = sqrt(3.0 * V) * P->eps;
-  P->res[0] = r1;
-  P->res[1] = r2;
-  P->tol[0] = t1;
-  P->tol[1] = t2;
-  P->iter += 1;
-  const int it = P->iter;
-  if (hist && it + P->iter_base <= hist_cap) {
-    double* h = hist + ((long long)p * hist_cap + (it + P->iter_base - 1)) * SOLUTE_HIST;
-    h[0] = r1;
-    h[1] = r2;
-    h[2] = t1;
-    h[3] = t2;
+  const int lane = threadIdx.x;
+  const bool first = threadIdx.x < 32;
+  double eps = 0, rmin = 0;
+  int max_iter = 0, iter = 0, iter_base = 0, stall_win = 0;
+  if (first) {
+    eps = P->eps;
+    rmin = P->rmin;
+    max_iter = P->max_iter;
+    iter = P->iter;
+    iter_base = P->iter_base;
+    stall_win = P->stall_win;
   }
-  const double rn = r1 / (1.0 + t1);
-  if (!(isfinite(r1) && isfinite(r2))) {
+  double v[FIN_VALS] = {0, 0, 0, 0, 0, 0, 0, 0};
+  add_partials<2>(part_z + (long long)p * nbz * 4, nbz, 4, v);
+  const double total = block_sum8(v, red);
+  if (!first) return;
+  // lane 0: r1 and its tolerance, lane 1: r2 (Eq. 19)
+  const double r = sqrt(total / V), t = sqrt((lane & 1) ? 3.0 * V : V) * eps;
+  const int it = iter + 1;
+  if (lane < 2) {
+    P->res[lane] = r;
+    P->tol[lane] = t;
+    if (hist && it + iter_base <= hist_cap) {
+      double* h = hist + ((long long)p * hist_cap + (it + iter_base - 1)) * SOLUTE_HIST;
+      h[lane] = r;
+      h[2 + lane] = t;
+    }
+  }
+  const bool finite = (__ballot_sync(0xffffffffu, isfinite(r)) & 3u) == 3u;
+  const bool conv = (__ballot_sync(0xffffffffu, r <= t) & 3u) == 3u;
+  const double q = stall_win > 0 ? (t > 0.0 ? r / t : r) : 0.0, q1 = shfl(q, 1);
+  if (lane != 0) return;
+  P->iter = it;
+  const double rn = r / (1.0 + t);
+  if (!finite) {
     P->done = 1;
     P->status = ST_NONFINITE;
     return;
   }
-  if (r1 <= t1 && r2 <= t2) {
+  if (conv) {
     P->done = 1;
     P->converged = 1;
     P->status = ST_OK;
     return;
   }
-  if (it > 20 && rn > 1e3 * P->rmin) {
+  if (it > 20 && rn > 1e3 * rmin) {
     P->done = 1;
     P->status = ST_DIVERGED;
     return;
   }
-  if (rn < P->rmin) P->rmin = rn;
-  const double rr[2] = {r1, r2}, tt[2] = {t1, t2};
-  if (stalled(P->stall_win, P->stall_n, P->stall_best, rr, tt, 2)) {
+  if (rn < rmin) P->rmin = rn;
+  if (stalled(stall_win, P->stall_n, P->stall_best, fmax(fmax(0.0, q), q1))) {
     P->done = 1;
     P->status = ST_STALLED;
     return;
   }
-  if (it >= P->max_iter) {
+  if (it >= max_iter) {
     P->done = 1;
     P->status = ST_MAXITER;
   }
@@ -213,15 +295,22 @@ cudaError_t loop_control(const LoopCtl& c, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// a thread of the finalize block takes about four records, in blocks of 128 to 1024
+static int fin_threads(int records) {
+  int t = 128;
+  while (t < 1024 && records > 4 * t) t *= 2;
+  return t;
+}
+
 cudaError_t stokes_finalize(int nprob, StokesDev* prm, const double* part_x, int nbx, const double* part_z,
                             int nbz, double V, double* hist, int hist_cap, cudaStream_t s) {
-  k_stokes_finalize<<<nprob, 256, 0, s>>>(prm, part_x, nbx, part_z, nbz, V, hist, hist_cap);
+  k_stokes_finalize<<<nprob, fin_threads(nbx > nbz ? nbx : nbz), 0, s>>>(prm, part_x, nbx, part_z, nbz, V, hist, hist_cap);
   return cudaGetLastError();
 }
 
 cudaError_t solute_finalize(int nprob, SoluteDev* prm, const double* part_z, int nbz, double V, double* hist,
                             int hist_cap, cudaStream_t s) {
-  k_solute_finalize<<<nprob, 256, 0, s>>>(prm, part_z, nbz, V, hist, hist_cap);
+  k_solute_finalize<<<nprob, fin_threads(nbz), 0, s>>>(prm, part_z, nbz, V, hist, hist_cap);
   return cudaGetLastError();
 }
 

@@ -51,6 +51,35 @@ __device__ __forceinline__ cx<T> mul_i(cx<T> a) { return mk<T>(-a.y, a.x); }
 template <typename T>
 __device__ __forceinline__ T cabs2(cx<T> a) { return a.x * a.x + a.y * a.y; }
 
+// Twiddle products with their contraction written out: which product of a complex
+// multiplication is rounded before the other is fused into it would otherwise be
+// the compiler's choice, and change from kernel to kernel. F = 0: the products
+// with a.y are rounded (forward transforms); F = 1: in the imaginary part the one
+// with a.x is (inverse ones).
+template <int F>
+__device__ __forceinline__ cx<float> cmul_fma(cx<float> a, cx<float> b) {
+  return mk<float>(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)),
+                   F == 0 ? __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)) : __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+template <int F>
+__device__ __forceinline__ cx<double> cmul_fma(cx<double> a, cx<double> b) {
+  return mk<double>(__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)),
+                    F == 0 ? __fma_rn(a.x, b.y, __dmul_rn(a.y, b.x)) : __fma_rn(a.y, b.x, __dmul_rn(a.x, b.y)));
+}
+
+// a product that is not contracted into a later addition
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// a b + c d with one product rounded: that of c d, or (SECOND) that of a b
+template <bool SECOND, typename T>
+__device__ __forceinline__ T sum2(T a, T b, T c, T d) {
+  return SECOND ? fma_rn(c, d, mul_rn(a, b)) : fma_rn(a, b, mul_rn(c, d));
+}
+
 // padded shared-memory index: one spare slot after every 16 elements
 __host__ __device__ constexpr int pad(int i) { return i + (i >> 4); }
 __host__ __device__ constexpr int ept(int n) { return n < 16 ? n : 16; }  // elements per thread

@@ -153,22 +153,6 @@ __device__ __forceinline__ cx<T> lp_tw(const cx<T>* __restrict__ twg, int e) {
   return w;
 }
 
-// Twiddle products with their contraction written out: which product of a complex
-// multiplication is rounded before the other is fused into it would otherwise be
-// the compiler's choice, and change from kernel to kernel. F = 0: the products
-// with a.y are rounded (forward transforms); F = 1: in the imaginary part the one
-// with a.x is (inverse ones).
-template <int F>
-__device__ __forceinline__ cx<float> cmul_fma(cx<float> a, cx<float> b) {
-  return mk<float>(__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)),
-                   F == 0 ? __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x)) : __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)));
-}
-template <int F>
-__device__ __forceinline__ cx<double> cmul_fma(cx<double> a, cx<double> b) {
-  return mk<double>(__fma_rn(a.x, b.x, -__dmul_rn(a.y, b.y)),
-                    F == 0 ? __fma_rn(a.x, b.y, __dmul_rn(a.y, b.x)) : __fma_rn(a.y, b.x, __dmul_rn(a.x, b.y)));
-}
-
 // Stages after the first, from span Ns on (see the head of the file). b: the
 // column's exchange buffer, holding the outputs of the previous stage.
 template <typename T, int N, int W, int Ns, int SIGN, int F>
@@ -289,19 +273,6 @@ __device__ __forceinline__ void lp_inverse_scaled(cx<float> (&v)[LCfg<float, N, 
     __syncthreads();
     lp_stage<float, N, W, C::E, +1, 1>(v, b, twg, t);
   }
-}
-
-// a product that is not contracted into a later addition
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-
-__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
-
-// a b + c d with one product rounded: that of c d, or (SECOND) that of a b
-template <bool SECOND, typename T>
-__device__ __forceinline__ T sum2(T a, T b, T c, T d) {
-  return SECOND ? fma_rn(c, d, mul_rn(a, b)) : fma_rn(a, b, mul_rn(c, d));
 }
 
 template <typename T, int E>

@@ -490,14 +490,26 @@ struct StokesGroup {
   int lph;
 };
 
+// Iterations per turn of the loop node: up to four where an iteration of all problems
+// takes tens of microseconds, preferably a divisor of the iteration cap.
+int loop_unroll(long long voxels, unsigned cap) {
+  if (voxels > (1LL << 22)) return 1;
+  for (int u : {4, 3, 2})
+    if (cap % u == 0) return u;
+  return cap >= 16 ? 4 : 1;
+}
+
 // Device-resident loop: a CUDA graph whose while node repeats the work that
 // `capture` enqueues (one iteration of every context in `ctxs`) followed by
 // the loop-control kernel, until every stop flag of `lc` is set or `cap`
 // iterations have run; the host launches it once and waits. The instantiated
 // graph is cached in `cache` while its key and the contexts' buffers stay the same.
+// The body holds `unroll` iterations before the control kernel: on small grids its
+// launch and the node's turn cost as much as a pass (an iteration that follows the
+// last one needed finds every stop flag set and returns at once).
 template <typename Capture>
 acm_status graph_loop_run(GraphCache& cache, const GraphKey& key, std::vector<acm_ctx*>& ctxs, Capture&& capture,
-                          LoopCtl lc, cudaStream_t st) {
+                          LoopCtl lc, cudaStream_t st, int unroll) {
   if (!(cache.exec && cache.key == key)) {
     if (cache.exec) {
       cudaGraphExecDestroy(cache.exec);
@@ -548,7 +560,9 @@ acm_status graph_loop_run(GraphCache& cache, const GraphKey& key, std::vector<ac
       cudaGetLastError();
       return ACM_ERR_CUDA;
     }
-    acm_status s = capture();
+    acm_status s = ACM_OK;
+    for (int i = 0; i < unroll && s == ACM_OK; ++i) s = capture();
+    lc.step = (unsigned)unroll;
     lc.counter = cache.counter;
     lc.cap = key.cap;
     lc.handle = handle;
@@ -597,6 +611,8 @@ acm_status stokes_graph_run(std::vector<StokesGroup>& grp, int deriv, unsigned c
   key.cap = cap;
   std::vector<acm_ctx*> ctxs;
   LoopCtl lc = {};
+  long long voxels = 0;
+  for (auto& x : grp) voxels += (long long)x.nprob * x.c->g.V;
   for (size_t i = 0; i < grp.size(); ++i) {
     ctxs.push_back(grp[i].c);
     lc.base[i] = (const char*)grp[i].c->sprm;
@@ -615,7 +631,7 @@ acm_status stokes_graph_run(std::vector<StokesGroup>& grp, int deriv, unsigned c
     }
     return s;
   };
-  return graph_loop_run(cache, key, ctxs, capture, lc, st);
+  return graph_loop_run(cache, key, ctxs, capture, lc, st, loop_unroll(voxels, cap));
 }
 
 // Iterations of the device-resident loop. With device_loop (and the profiler
@@ -943,7 +959,7 @@ acm_status solute_run(acm_ctx* c, int nprob, const uint8_t* Hdev, const void* ud
     lc.ngroups = 1;
     lc.done_off = (int)offsetof(SoluteDev, done);
     auto capture = [&]() -> acm_status { return solute_body<T>(c, nprob, Hdev, udev, us, sym); };
-    return graph_loop_run(c->graph_sol, key, ctxs, capture, lc, c->st);
+    return graph_loop_run(c->graph_sol, key, ctxs, capture, lc, c->st, loop_unroll((long long)nprob * g.V, key.cap));
   }
   // host-launched chunks of check_every iterations; the stop flags are read between chunks
   CKS(pin_scratch(c, (size_t)c->B * sizeof(SoluteDev)));

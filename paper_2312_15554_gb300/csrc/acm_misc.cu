@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(256) k_loop_control(LoopCtl c) {
   if (mine) any = 1;
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned int it = *c.counter + 1;
+    const unsigned int it = *c.counter + c.step;
     *c.counter = it;
     cudaGraphSetConditional(c.handle, (any && it < c.cap) ? 1u : 0u);
   }

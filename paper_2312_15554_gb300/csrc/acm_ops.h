@@ -82,6 +82,7 @@ struct LoopCtl {
   int done_off;
   unsigned int* counter;  // iterations run so far (device)
   unsigned int cap;
+  unsigned int step;      // iterations per turn
   cudaGraphConditionalHandle handle;
 };
 cudaError_t loop_control(const LoopCtl& c, cudaStream_t s);

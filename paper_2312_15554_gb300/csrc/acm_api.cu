@@ -438,6 +438,7 @@ acm_status stokes_setup(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs
     d.max_iter = P.max_iter;
     d.stall_win = stall_win;
     d.stall_best = 1e300;
+    d.b_next = d.psi[2];
     if (preset_status && preset_status[p] != ACM_OK) {  // degenerate cell: not iterated
       d.done = 1;
       d.status = preset_status[p];
@@ -448,37 +449,39 @@ acm_status stokes_setup(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs
   return ACM_OK;
 }
 
-// step 1 of the coming iteration (Eq. 7 / Eq. 13): w -> u^ -> u (up to the x-pass)
+// the right-hand side of Eq. 7 along x, for the problems that do not have it in place
 template <typename T>
-acm_status stokes_step1(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs, int lph, const Sym<T>& sym) {
+acm_status stokes_rhs(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs, int lph) {
+  Prec& w = prec<T>(c);
+  Geo g = c->g;
+  g.hs = hs;
+  g.lph = lph;
+  LK(ACM_K_X_STOKES_RHS, Ops<T>::x_stokes_rhs(g, nprob, w.spec, w.u, w.lam, Hdev, c->Hb, c->sprm, w.tw, c->st));
+  return ACM_OK;
+}
+
+// One ADMM iteration of nprob problems whose right-hand side is in place: step 1
+// (Eq. 7 / Eq. 13), then steps 2-4 (x pass, which leaves the next right-hand side,
+// and finalize). `repair` (adaptive penalties, not the last iteration): the x pass
+// again where Eq. 22 gave another b than it was formed with.
+template <typename T>
+acm_status stokes_body(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs, int lph, const Sym<T>& sym,
+                       bool repair) {
   Prec& w = prec<T>(c);
   Geo g = c->g;
   g.hs = hs;
   g.lph = lph;
   const long long ps = 3 * g.S;
-  LK(ACM_K_X_STOKES_RHS, Ops<T>::x_stokes_rhs(g, nprob, w.spec, w.u, w.lam, Hdev, c->Hb, c->sprm, w.tw, c->st));
-  LK(ACM_K_Y_FWD_STOKES, Ops<T>::pass(g, 1, P_FWD, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, c->sprm, nullptr, nullptr, c->st));
-  LK(ACM_K_Z_STOKES, Ops<T>::pass(g, 0, P_STOKES, 3, nprob, w.spec, ps, sym, w.tw, w.st0, w.st1, c->sprm, nullptr, c->part_z, c->st));
-  LK(ACM_K_Y_INV_STOKES, Ops<T>::pass(g, 1, P_INV, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, c->sprm, nullptr, nullptr, c->st));
-  return ACM_OK;
-}
-
-// One ADMM iteration of nprob problems after the previous one's step 1:
-// steps 2-4 (x pass + finalize), then step 1 of the next iteration.
-template <typename T>
-acm_status stokes_body(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs, int lph, const Sym<T>& sym,
-                       bool last) {
-  Prec& w = prec<T>(c);
-  Geo g = c->g;
-  g.hs = hs;
-  g.lph = lph;
   const int nbx = Ops<T>::x_blocks(g), nbz = Ops<T>::z_blocks(g, P_STOKES);
   double* hist = c->hist_b ? c->hist_b : (nprob <= BMAX ? c->hist : nullptr);
   const int hcap = c->hist_b ? c->hist_b_cap : HIST_CAP;
+  LK(ACM_K_Y_FWD_STOKES, Ops<T>::pass(g, 1, P_FWD, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, c->sprm, nullptr, nullptr, c->st));
+  LK(ACM_K_Z_STOKES, Ops<T>::pass(g, 0, P_STOKES, 3, nprob, w.spec, ps, sym, w.tw, w.st0, w.st1, c->sprm, nullptr, c->part_z, c->st));
+  LK(ACM_K_Y_INV_STOKES, Ops<T>::pass(g, 1, P_INV, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, c->sprm, nullptr, nullptr, c->st));
   LK(ACM_K_X_STOKES_LOCAL, Ops<T>::x_stokes_local(g, nprob, w.spec, w.u, w.lam, Hdev, c->Hb, c->sprm, c->part_x, w.tw,
                                                   c->st));
   LK(ACM_K_FINALIZE, stokes_finalize(nprob, c->sprm, c->part_x, nbx, c->part_z, nbz, (double)g.V, hist, hcap, c->st));
-  if (!last) CKS(stokes_step1<T>(c, nprob, Hdev, hs, lph, sym));
+  if (repair) CKS(stokes_rhs<T>(c, nprob, Hdev, hs, lph));
   return ACM_OK;
 }
 
@@ -598,9 +601,10 @@ acm_status graph_loop_run(GraphCache& cache, const GraphKey& key, std::vector<ac
   return ACM_OK;
 }
 
-// The Stokes loop of every group as one device-resident graph: [step 1, steps 2-4].
+// The Stokes loop of every group as one device-resident graph, after the first
+// right-hand sides.
 template <typename T>
-acm_status stokes_graph_run(std::vector<StokesGroup>& grp, int deriv, unsigned cap, GraphCache& cache,
+acm_status stokes_graph_run(std::vector<StokesGroup>& grp, int deriv, bool adaptive, unsigned cap, GraphCache& cache,
                             cudaStream_t st) {
   GraphKey key;
   key.prec = (int)sizeof(T);
@@ -609,6 +613,7 @@ acm_status stokes_graph_run(std::vector<StokesGroup>& grp, int deriv, unsigned c
   key.deriv = deriv;
   key.kind = 1;
   key.cap = cap;
+  key.kx = adaptive;
   std::vector<acm_ctx*> ctxs;
   LoopCtl lc = {};
   long long voxels = 0;
@@ -626,11 +631,11 @@ acm_status stokes_graph_run(std::vector<StokesGroup>& grp, int deriv, unsigned c
     for (size_t i = 0; i < grp.size() && s == ACM_OK; ++i) {
       StokesGroup& x = grp[i];
       const Sym<T> sym = sym_of<T>(x.c, deriv);
-      s = stokes_step1<T>(x.c, x.nprob, x.H, x.hs, x.lph, sym);
-      if (s == ACM_OK) s = stokes_body<T>(x.c, x.nprob, x.H, x.hs, x.lph, sym, true);
+      s = stokes_body<T>(x.c, x.nprob, x.H, x.hs, x.lph, sym, adaptive);
     }
     return s;
   };
+  for (StokesGroup& x : grp) CKS(stokes_rhs<T>(x.c, x.nprob, x.H, x.hs, x.lph));
   return graph_loop_run(cache, key, ctxs, capture, lc, st, loop_unroll(voxels, cap));
 }
 
@@ -640,20 +645,20 @@ acm_status stokes_graph_run(std::vector<StokesGroup>& grp, int deriv, unsigned c
 // launches past `remaining`; problems that converge earlier turn the rest of
 // their launches into immediate returns.
 template <typename T>
-acm_status stokes_iterate(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs, int lph, int deriv,
+acm_status stokes_iterate(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs, int lph, int deriv, bool adaptive,
                           int check_every, int remaining, bool device_loop) {
   if (remaining <= 0) return ACM_OK;
   if (device_loop && !c->prof) {
     std::vector<StokesGroup> grp = {{c, nprob, Hdev, hs, lph}};
-    return stokes_graph_run<T>(grp, deriv, (unsigned)remaining, c->graph, c->st);
+    return stokes_graph_run<T>(grp, deriv, adaptive, (unsigned)remaining, c->graph, c->st);
   }
   const Sym<T> sym = sym_of<T>(c, deriv);
-  CKS(stokes_step1<T>(c, nprob, Hdev, hs, lph, sym));
+  CKS(stokes_rhs<T>(c, nprob, Hdev, hs, lph));
   CKS(pin_scratch(c, (size_t)c->B * sizeof(StokesDev)));
   if (check_every < 1) check_every = 1;
   while (remaining > 0) {
     const int chunk = check_every < remaining ? check_every : remaining;
-    for (int k = 0; k < chunk; ++k) CKS(stokes_body<T>(c, nprob, Hdev, hs, lph, sym, remaining - k <= 1));
+    for (int k = 0; k < chunk; ++k) CKS(stokes_body<T>(c, nprob, Hdev, hs, lph, sym, adaptive && remaining - k > 1));
     remaining -= chunk;
     CK(cudaMemcpyAsync(c->pin, c->sprm, nprob * sizeof(StokesDev), cudaMemcpyDeviceToHost, c->st));
     CK(cudaStreamSynchronize(c->st));
@@ -684,6 +689,7 @@ acm_status stokes_promote(acm_ctx* c, int nprob, double eps) {
     x.status = 0;
     x.eps = eps;
     x.stall_win = 0;
+    x.rhs_ok = 0;  // the spectra in place are FP32 ones
   }
   CK(cudaMemcpyAsync(c->sprm, hp.data(), nprob * sizeof(StokesDev), cudaMemcpyHostToDevice, c->st));
   return ACM_OK;
@@ -797,12 +803,12 @@ acm_status stokes_solve(acm_ctx* c, int nprob, const uint8_t* H, const double (*
   const std::vector<const void*> iu(nprob, init_u), il(nprob, init_lam);
   if (P.precision == ACM_FP32) {
     CKS(stokes_setup<float>(c, nprob, Hdev, 0, 1, gs, P, P.eps, iu.data(), il.data(), nullptr, 0, pore_l.data()));
-    CKS(stokes_iterate<float>(c, nprob, Hdev, 0, 1, P.deriv, P.check_every, P.max_iter, dl));
+    CKS(stokes_iterate<float>(c, nprob, Hdev, 0, 1, P.deriv, P.adaptive != 0, P.check_every, P.max_iter, dl));
     CKS(stokes_outputs<float>(c, nprob, u_out, u_stride, p_out, lam_out, Kcol));
     st = stokes_reports(c, nprob, rep, -1, t0);
   } else if (P.precision == ACM_FP64) {
     CKS(stokes_setup<double>(c, nprob, Hdev, 0, 1, gs, P, P.eps, iu.data(), il.data(), nullptr, 0, pore_l.data()));
-    CKS(stokes_iterate<double>(c, nprob, Hdev, 0, 1, P.deriv, P.check_every, P.max_iter, dl));
+    CKS(stokes_iterate<double>(c, nprob, Hdev, 0, 1, P.deriv, P.adaptive != 0, P.check_every, P.max_iter, dl));
     CKS(stokes_outputs<double>(c, nprob, u_out, u_stride, p_out, lam_out, Kcol));
     st = stokes_reports(c, nprob, rep, -2, t0);
   } else {
@@ -811,7 +817,7 @@ acm_status stokes_solve(acm_ctx* c, int nprob, const uint8_t* H, const double (*
     if (init_u || init_lam) return ACM_ERR_ARG;  // warm starts are taken in the FP32 or FP64 modes
     CKS(stokes_setup<float>(c, nprob, Hdev, 0, 1, gs, P, e32, nullptr, nullptr, nullptr, STALL_WINDOW,
                             pore_l.data()));
-    CKS(stokes_iterate<float>(c, nprob, Hdev, 0, 1, P.deriv, P.check_every, P.max_iter, dl));
+    CKS(stokes_iterate<float>(c, nprob, Hdev, 0, 1, P.deriv, P.adaptive != 0, P.check_every, P.max_iter, dl));
     std::vector<StokesDev> hp(nprob);
     CK(cudaMemcpy(hp.data(), c->sprm, nprob * sizeof(StokesDev), cudaMemcpyDeviceToHost));
     // FP32 iterations of each problem; the host loop may run until the problem
@@ -827,7 +833,7 @@ acm_status stokes_solve(acm_ctx* c, int nprob, const uint8_t* H, const double (*
     }
     if (ok && P.eps < e32) {
       CKS(stokes_promote(c, nprob, P.eps));
-      CKS(stokes_iterate<double>(c, nprob, Hdev, 0, 1, P.deriv, P.check_every, P.max_iter - it32_min, dl));
+      CKS(stokes_iterate<double>(c, nprob, Hdev, 0, 1, P.deriv, P.adaptive != 0, P.check_every, P.max_iter - it32_min, dl));
       CKS(stokes_outputs<double>(c, nprob, u_out, u_stride, p_out, lam_out, Kcol));
       st = stokes_reports(c, nprob, rep, 0, t0, &it32);
     } else {
@@ -1240,10 +1246,10 @@ acm_status batch_stokes_run(acm_batch* b, const uint8_t* const* H, const acm_sto
   bool prof = false;
   for (auto& gr : b->groups) prof = prof || gr.c->prof;
   if (P.device_loop && !prof) {
-    CKS(stokes_graph_run<T>(grp, P.deriv, (unsigned)P.max_iter, b->graph, b->st));
+    CKS(stokes_graph_run<T>(grp, P.deriv, P.adaptive != 0, (unsigned)P.max_iter, b->graph, b->st));
   } else {
     for (auto& x : grp)
-      CKS(stokes_iterate<T>(x.c, x.nprob, x.H, x.hs, x.lph, P.deriv, P.check_every, P.max_iter, false));
+      CKS(stokes_iterate<T>(x.c, x.nprob, x.H, x.hs, x.lph, P.deriv, P.adaptive != 0, P.check_every, P.max_iter, false));
   }
   // outputs: K per cell (volume averages of the three loads), fields, reports
   const double t1 = now_ms();

@@ -1,11 +1,14 @@
 // acm_kernels.cuh -- the ACM hot path as fused FFT-pass kernels (sm_103a).
 //
-// One Stokes ADMM iteration (Section 3.1) is five pass kernels plus a tiny
+// One Stokes ADMM iteration (Section 3.1) is four pass kernels plus a tiny
 // FP64 finalize kernel:
 //   x_stokes_local   C2R along x of u^{n+1}, steps 2-3 (Eq. 8-9) pointwise,
-//                    partial sums of the Eq. 10 residuals
+//                    partial sums of the Eq. 10 residuals, and w = b u~ - a (the
+//                    known part of Eq. 7) with the penalty b that Eq. 22 is
+//                    expected to give, R2C along x
 //   stokes_finalize  residuals, tolerances (Eq. 11-12), stop test, Eq. 22
-//   x_stokes_rhs     w = b u~ - a (the known part of Eq. 7), R2C along x
+//   x_stokes_rhs     w and its R2C again where b came out otherwise (and before
+//                    the first iteration)
 //   strided<FWD>     forward FFT along y
 //   strided<STOKES>  forward FFT along z, Eq. 13 solve per wavevector, q update
 //                    of Eq. 9 in Fourier space, divergence residuals by
@@ -179,16 +182,22 @@ __host__ constexpr XGrid xs_grid(int groups) {
 }
 
 // ---------------------------------------------------------------------------
-// Stokes x-pass 1: C2R of u^{n+1}, steps 2-3 of ADMM, residual partial sums
+// Stokes x-pass 1: C2R of u^{n+1}, steps 2-3 of ADMM, residual partial sums, and
+// the right-hand side of the next Eq. 7 with its R2C
 //
 // Line-resident: each component of a line is inverse-transformed into
 // registers and the local steps run on the lane's voxel pairs 2k, 2k+1 read
 // and written as vectors; a chunk of pairs loads its old state before it
-// stores, so no store waits for the load of its own address.
+// stores, so no store waits for the load of its own address. The new u and lambda
+// are in registers then, so w = b u~ - a is formed and transformed forward there: a
+// pass of its own read both fields again (283 us a launch at 256^3 and three
+// problems, beside 554 for this kernel). The penalty b of the next iteration follows
+// from residuals that are complete only after the launch; b_next guesses it, and
+// x_stokes_rhs repairs a wrong guess.
 // ---------------------------------------------------------------------------
 template <typename T, int N2>
 __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
-    k_x_stokes_local(const cx<T>* __restrict__ spec, T* __restrict__ u, T* __restrict__ lam,
+    k_x_stokes_local(cx<T>* __restrict__ spec, T* __restrict__ u, T* __restrict__ lam,
                      const uint8_t* __restrict__ H, const uint32_t* __restrict__ Hb, StokesDev* __restrict__ prm,
                      double* __restrict__ part, Geo g, const cx<T>* __restrict__ twg, int gpw) {
   using L = XL<T, N2>;
@@ -200,7 +209,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   cx<T>* tw = reinterpret_cast<cx<T>*>(smem_raw);
   cx<T>* lines = tw + xs_tw_slots<T, N2>();
   __shared__ T red[5 * 32];
-  __shared__ T kpar[3];
+  __shared__ T kpar[5];
   const int p = blockIdx.y;
   // components of this block: all three, or one each (see xs_grid)
   const int cb = blockIdx.z, ce = gridDim.z == 1 ? 3 : cb + 1;
@@ -213,8 +222,12 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     kpar[0] = (T)P->psi[0];
     kpar[1] = (T)P->psi[2];
     kpar[2] = (T)(P->psi_prev[2] / (P->psi_prev[2] + P->psi_prev[0]));
+    // the next right-hand side: its penalty, and u~ = s_rhs u on solid voxels
+    kpar[3] = (T)P->b_next;
+    kpar[4] = (T)(P->psi[2] / (P->psi[2] + P->psi[0]));
   }
   __syncthreads();
+  const T b_rhs = kpar[3], s_rhs = kpar[4];
   const T alpha = kpar[0], b = kpar[1];
   const T s_prev = kpar[2];
   const T s_now = b / (b + alpha);
@@ -223,7 +236,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   const unsigned mask = xl_mask();
   cx<T>* b0 = lines + (warp * LPW + ll) * LB;
   cx<T>* b1 = b0 + LS;
-  const cx<T>* sp = spec + (long long)p * 3 * g.S;
+  cx<T>* sp = spec + (long long)p * 3 * g.S;
   T* up = u + (long long)p * 3 * g.V;
   T* lp = lam + (long long)p * 3 * g.V;
   const long long hcell = (long long)(p / g.lph) * g.hs;
@@ -239,7 +252,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
     if (grp >= ngroups) break;
     const long long line = (long long)grp * LPW + ll;
     const long long v0 = line * N2;
-    const cx<T>* srow = sp + line * g.P;
+    cx<T>* srow = sp + line * g.P;
     __syncwarp(mask);
     for (int e = t; e <= M; e += TL) {
       cp_async<(int)sizeof(cx<T>)>(&b0[pad(e)], &srow[cb * g.S + e]);
@@ -297,8 +310,8 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
           *reinterpret_cast<T2*>(uc + 2 * k) = w;
           const T dua = u1a - u0[j].x, dub = u1b - u0[j].y;
           a3 += dua * dua + dub * dub;
+          T2 ln = l0[j];
           if (sa | sb) {
-            T2 ln = l0[j];
             if (sa) {
               const T ut1 = s_now * u1a, ut0 = s_prev * u0[j].x;   // step 2 (Eq. 8) with a^n = H lambda^n
               ln.x = l0[j].x + alpha * ut1;                          // step 3 (Eq. 9)
@@ -319,16 +332,12 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
             }
             *reinterpret_cast<T2*>(lc + 2 * k) = ln;   // lambda stays 0 on pore voxels
           }
+          // Eq. 7 right-hand side w = b u~ - a with a = H lambda, as in k_x_stokes_rhs
+          v[m] = mk<T>(sa ? b_rhs * (s_rhs * u1a) - ln.x : b_rhs * u1a, sb ? b_rhs * (s_rhs * u1b) - ln.y : b_rhs * u1b);
         }
       };
       load_chunk(0, ua, la);
       xl_inverse<T, N2>(bc, tw, t, mask, v);
-      if (c == cb && ce == cb + 3) {
-        // the row of component 2 into b0, behind components 0 and 1
-        __syncwarp(mask);
-        for (int e = t; e <= M; e += TL) cp_async<(int)sizeof(cx<T>)>(&b0[pad(e)], &srow[2 * g.S + e]);
-        cp_async_commit();
-      }
       // rolling: chunk j + 1 travels while chunk j is stepped
 #pragma unroll
       for (int j = 0; j < E / CH; ++j) {
@@ -339,7 +348,18 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
         if (j & 1) step_chunk(j * CH, ub, lb);
         else step_chunk(j * CH, ua, la);
       }
-      if (c == cb + 1) {
+      cx<T> xn;
+      xl_forward<T, N2>(bc, tw, t, mask, v, v, xn);
+      cx<T>* dst = srow + c * g.S;
+#pragma unroll
+      for (int m = 0; m < E; ++m) dst[t + TL * m] = v[m];
+      if (t == 0) dst[M] = xn;
+      if (c == cb && ce == cb + 3) {
+        // the row of component 2 into b0, behind component 1
+        __syncwarp(mask);
+        for (int e = t; e <= M; e += TL) cp_async<(int)sizeof(cx<T>)>(&b0[pad(e)], &srow[2 * g.S + e]);
+        cp_async_commit();
+      } else if (c == cb + 1) {
         cp_async_wait<0>();
         __syncwarp(mask);
       }
@@ -354,7 +374,9 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
 }
 
 // ---------------------------------------------------------------------------
-// Stokes x-pass 2: w = b u~ - a (Eq. 7 right-hand side), R2C along x
+// Stokes x-pass 2: w = b u~ - a (Eq. 7 right-hand side), R2C along x, for the
+// problems whose right-hand side is not in place (before the first iteration, and
+// after a wrong guess of b)
 // ---------------------------------------------------------------------------
 template <typename T, int N2>
 __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
@@ -374,7 +396,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32, sizeof(T) == 4 ? 2 : 1)
   // components of this block: all three, or one each (see xs_grid)
   const int cb = blockIdx.z, ce = gridDim.z == 1 ? 3 : cb + 1;
   const StokesDev* P = prm + p;
-  if (P->done) return;
+  if (P->done || P->rhs_ok) return;
   xl_load_tw<T, N2, TW_MAX>(tw, twg);
   if (threadIdx.x == 0) {
     // converted once per block; u~^n on solid voxels = s_prev u^n with the

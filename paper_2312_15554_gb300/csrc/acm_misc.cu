@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(1024) k_stokes_finalize(StokesDev* __restrict_
   // warp 0 reads the control block while the partial sums travel: lane k holds
   // entry k of the vectors
   const int k3 = lane < 3 ? lane : 0;
-  double psi = 0, phi = 0, tau = 0, psi_min = 0, mean = 0, e = 0;
+  double psi = 0, phi = 0, tau = 0, psi_min = 0, mean = 0, e = 0, b_next = 0;
   int adaptive = 0, max_iter = 0, iter = 0, iter_base = 0, stall_win = 0;
   if (first) {
     psi = P->psi[k3];
@@ -98,6 +98,7 @@ __global__ void __launch_bounds__(1024) k_stokes_finalize(StokesDev* __restrict_
     psi_min = P->psi_min[k3];
     mean = P->mean_u[k3];
     e = P->eps;
+    b_next = P->b_next;
     adaptive = P->adaptive;
     max_iter = P->max_iter;
     iter = P->iter;
@@ -147,9 +148,20 @@ __global__ void __launch_bounds__(1024) k_stokes_finalize(StokesDev* __restrict_
   if (lane < 3) {
     P->psi_last[lane] = psi;
     P->psi_prev[lane] = psi;
+    double next = psi, guess = psi;  // guess: the change of this iteration once more
     if (adaptive) {  // Eq. 22: pair k drives (alpha, beta, b)[k]
-      if (rp > tau * rd) P->psi[lane] = phi * psi;
-      else if (rd > tau * rp) P->psi[lane] = fmax(psi / phi, psi_min);
+      if (rp > tau * rd) {
+        next = phi * psi;
+        guess = phi * next;
+      } else if (rd > tau * rp) {
+        next = fmax(psi / phi, psi_min);
+        guess = fmax(next / phi, psi_min);
+      }
+      P->psi[lane] = next;
+    }
+    if (lane == 2) {
+      P->rhs_ok = next == b_next;
+      P->b_next = guess;
     }
   }
   double m = 0.0;

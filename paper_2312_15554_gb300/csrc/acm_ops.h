@@ -23,7 +23,7 @@ struct Ops {
   static int pass_tx(const Geo& g, int axis, int op, int nc);
   static bool tx_variant(int n, int op, int nc, int shift);
 
-  static cudaError_t x_stokes_local(const Geo& g, int nprob, const void* spec, void* u, void* lam,
+  static cudaError_t x_stokes_local(const Geo& g, int nprob, void* spec, void* u, void* lam,
                                     const uint8_t* H, const uint32_t* Hb, StokesDev* prm, double* part,
                                     const void* tw, cudaStream_t s);
   static cudaError_t x_stokes_rhs(const Geo& g, int nprob, void* spec, const void* u, const void* lam,

@@ -51,14 +51,14 @@ static cudaError_t set_smem(K* k, int bytes) {
   }
 
 template <typename T, int N2>
-static cudaError_t l_x_local(const Geo& g, int nprob, const void* spec, void* u, void* lam, const uint8_t* H,
+static cudaError_t l_x_local(const Geo& g, int nprob, void* spec, void* u, void* lam, const uint8_t* H,
                              const uint32_t* Hb, StokesDev* prm, double* part, const void* tw, cudaStream_t s) {
   constexpr int smem = xs_smem_bytes<T, N2, 2, 0>();
   static const cudaError_t attr = set_smem(k_x_stokes_local<T, N2>, smem);
   if (attr != cudaSuccess) return attr;
   const XGrid x = xs_grid(g.n0 * g.n1 / XL<T, N2>::LPW);
   k_x_stokes_local<T, N2><<<dim3(x.blocks, nprob, x.csplit), x.warps * 32, xs_smem_bytes<T, N2, 2, 0>(x.warps), s>>>(
-      (const cx<T>*)spec, (T*)u, (T*)lam, H, Hb, prm, part, g, (const cx<T>*)tw, x.gpw);
+      (cx<T>*)spec, (T*)u, (T*)lam, H, Hb, prm, part, g, (const cx<T>*)tw, x.gpw);
   return cudaGetLastError();
 }
 
@@ -399,7 +399,7 @@ int Ops<T>::z_blocks(const Geo& g, int op) {
 }
 
 template <typename T>
-cudaError_t Ops<T>::x_stokes_local(const Geo& g, int nprob, const void* spec, void* u, void* lam, const uint8_t* H,
+cudaError_t Ops<T>::x_stokes_local(const Geo& g, int nprob, void* spec, void* u, void* lam, const uint8_t* H,
                                    const uint32_t* Hb, StokesDev* prm, double* part, const void* tw, cudaStream_t s) {
   ACM_DISPATCH_N(g.n2, l_x_local, g, nprob, spec, u, lam, H, Hb, prm, part, tw, s)
 }

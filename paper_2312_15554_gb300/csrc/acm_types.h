@@ -29,6 +29,11 @@ struct StokesDev {
   // its best value for stall_win iterations (its FP32 rounding floor)
   int stall_win, stall_n;
   double stall_best;
+  // The x pass forms the right-hand side of the coming iteration with b_next, a
+  // guess of the penalty b that Eq. 22 will give (the last change repeated);
+  // rhs_ok: the guess was right, so the spectra in place are that right-hand side
+  double b_next;
+  int rhs_ok;
 };
 
 struct SoluteDev {

@@ -475,9 +475,13 @@ acm_status stokes_body(acm_ctx* c, int nprob, const uint8_t* Hdev, long long hs,
   const int nbx = Ops<T>::x_blocks(g), nbz = Ops<T>::z_blocks(g, P_STOKES);
   double* hist = c->hist_b ? c->hist_b : (nprob <= BMAX ? c->hist : nullptr);
   const int hcap = c->hist_b ? c->hist_b_cap : HIST_CAP;
-  LK(ACM_K_Y_FWD_STOKES, Ops<T>::pass(g, 1, P_FWD, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, c->sprm, nullptr, nullptr, c->st));
-  LK(ACM_K_Z_STOKES, Ops<T>::pass(g, 0, P_STOKES, 3, nprob, w.spec, ps, sym, w.tw, w.st0, w.st1, c->sprm, nullptr, c->part_z, c->st));
-  LK(ACM_K_Y_INV_STOKES, Ops<T>::pass(g, 1, P_INV, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, c->sprm, nullptr, nullptr, c->st));
+  if (Ops<T>::plane_pass(g) >= 0) {
+    LK(ACM_K_Z_STOKES, Ops<T>::plane_stokes(g, nprob, w.spec, ps, sym, w.tw, w.st0, w.st1, c->sprm, c->part_z, c->st));
+  } else {
+    LK(ACM_K_Y_FWD_STOKES, Ops<T>::pass(g, 1, P_FWD, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, c->sprm, nullptr, nullptr, c->st));
+    LK(ACM_K_Z_STOKES, Ops<T>::pass(g, 0, P_STOKES, 3, nprob, w.spec, ps, sym, w.tw, w.st0, w.st1, c->sprm, nullptr, c->part_z, c->st));
+    LK(ACM_K_Y_INV_STOKES, Ops<T>::pass(g, 1, P_INV, 3, nprob, w.spec, ps, sym, w.tw, nullptr, nullptr, c->sprm, nullptr, nullptr, c->st));
+  }
   LK(ACM_K_X_STOKES_LOCAL, Ops<T>::x_stokes_local(g, nprob, w.spec, w.u, w.lam, Hdev, c->Hb, c->sprm, c->part_x, w.tw,
                                                   c->st));
   LK(ACM_K_FINALIZE, stokes_finalize(nprob, c->sprm, c->part_x, nbx, c->part_z, nbz, (double)g.V, hist, hcap, c->st));
@@ -1467,6 +1471,47 @@ acm_status ctx_create(acm_ctx** out, int n0, int n1, int n2, void* stream, int B
   return ACM_OK;
 }
 
+// The transforms of fft_impl in one precision. The strided passes run on the
+// context's spectrum; along axis 0 they read or write the caller's array itself when
+// it is a device buffer aligned to a complex element, else through a pitched copy.
+template <typename T>
+acm_status fft_run(acm_ctx* c, int nbatch, const void* in, void* out, bool forward) {
+  CKS(ensure_aux<T>(c));
+  const Geo& g = c->g;
+  const size_t rs = sizeof(T), cs = 2 * sizeof(T), spec = (size_t)g.n0 * g.n1 * g.Pu;
+  Prec& w = prec<T>(c);
+  const Sym<T> sym = sym_of<T>(c, 0);
+  const bool in_dev = is_device_ptr(in), out_dev = is_device_ptr(out);
+  const void* cplx = forward ? out : in;
+  const bool direct = (forward ? out_dev : in_dev) && (uintptr_t)cplx % cs == 0;
+  for (int b = 0; b < nbatch; ++b) {
+    const char* src = (const char*)in + (size_t)b * (forward ? g.V * rs : spec * cs);
+    char* dst = (char*)out + (size_t)b * (forward ? spec * cs : g.V * rs);
+    if (forward) {
+      const void* x = src;
+      if (!in_dev) {
+        CK(cudaMemcpyAsync(w.aux, src, g.V * rs, cudaMemcpyHostToDevice, c->st));
+        x = w.aux;
+      }
+      if ((uintptr_t)x % cs == 0) LK(ACM_K_OTHER, Ops<T>::x_r2c_lr(g, w.st0, x, w.tw, c->st));
+      else LK(ACM_K_OTHER, Ops<T>::x_r2c(g, 1, 1, w.st0, g.S, x, g.V, w.tw, c->st));
+      LK(ACM_K_OTHER, Ops<T>::pass(g, 1, P_FWD, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
+      LK(ACM_K_OTHER, Ops<T>::fft_z(g, false, w.st0, g.P, direct ? (void*)dst : w.st0, direct ? g.Pu : g.P, w.tw, c->st));
+      if (!direct)
+        CK(cudaMemcpy2DAsync(dst, g.Pu * cs, w.st0, g.P * cs, g.Pu * cs, (size_t)g.n0 * g.n1, cudaMemcpyDefault, c->st));
+    } else {
+      if (!direct)
+        CK(cudaMemcpy2DAsync(w.st0, g.P * cs, src, g.Pu * cs, g.Pu * cs, (size_t)g.n0 * g.n1, cudaMemcpyDefault, c->st));
+      LK(ACM_K_OTHER, Ops<T>::fft_z(g, true, direct ? (const void*)src : w.st0, direct ? g.Pu : g.P, w.st0, g.P, w.tw, c->st));
+      LK(ACM_K_OTHER, Ops<T>::pass(g, 1, P_INV, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
+      LK(ACM_K_OTHER, Ops<T>::x_c2r(g, 1, 1, w.st0, g.S, out_dev ? (void*)dst : w.aux, g.V, w.tw, c->st));
+      if (!out_dev) CK(cudaMemcpyAsync(dst, w.aux, g.V * rs, cudaMemcpyDeviceToHost, c->st));
+    }
+  }
+  CK(cudaStreamSynchronize(c->st));
+  return ACM_OK;
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -1598,54 +1643,7 @@ acm_status acm_advdiff_tensor(acm_ctx* c, const uint8_t* H, const void* u, doubl
 
 static acm_status fft_impl(acm_ctx* c, int fp64, int nbatch, const void* in, void* out, bool forward) {
   if (!c || !in || !out || nbatch < 1 || (fp64 != 0 && fp64 != 1)) return ACM_ERR_ARG;
-  const Geo& g = c->g;
-  const size_t rs = fp64 ? sizeof(double) : sizeof(float);
-  const size_t cs = 2 * rs;
-  if (fp64) CKS(ensure_aux<double>(c));
-  else CKS(ensure_aux<float>(c));
-  Prec& w = fp64 ? c->pd : c->pf;
-  for (int b = 0; b < nbatch; ++b) {
-    if (forward) {
-      const void* src = (const char*)in + (size_t)b * g.V * rs;
-      if (!is_device_ptr(in)) {
-        CK(cudaMemcpyAsync(w.aux, src, g.V * rs, cudaMemcpyHostToDevice, c->st));
-        src = w.aux;
-      }
-      if (fp64) {
-        const Sym<double> sym = sym_of<double>(c, 0);
-        LK(ACM_K_OTHER, Ops<double>::x_r2c(g, 1, 1, w.st0, g.S, src, g.V, w.tw, c->st));
-        LK(ACM_K_OTHER, Ops<double>::pass(g, 1, P_FWD, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
-        LK(ACM_K_OTHER, Ops<double>::pass(g, 0, P_FWD, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
-      } else {
-        const Sym<float> sym = sym_of<float>(c, 0);
-        LK(ACM_K_OTHER, Ops<float>::x_r2c(g, 1, 1, w.st0, g.S, src, g.V, w.tw, c->st));
-        LK(ACM_K_OTHER, Ops<float>::pass(g, 1, P_FWD, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
-        LK(ACM_K_OTHER, Ops<float>::pass(g, 0, P_FWD, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
-      }
-      CK(cudaMemcpy2DAsync((char*)out + (size_t)b * g.n0 * g.n1 * g.Pu * cs, g.Pu * cs, w.st0, g.P * cs, g.Pu * cs,
-                           (size_t)g.n0 * g.n1, cudaMemcpyDefault, c->st));
-    } else {
-      CK(cudaMemcpy2DAsync(w.st0, g.P * cs, (const char*)in + (size_t)b * g.n0 * g.n1 * g.Pu * cs, g.Pu * cs,
-                           g.Pu * cs, (size_t)g.n0 * g.n1, cudaMemcpyDefault, c->st));
-      void* dst = (char*)out + (size_t)b * g.V * rs;
-      const bool dev = is_device_ptr(out);
-      void* tgt = dev ? dst : w.aux;
-      if (fp64) {
-        const Sym<double> sym = sym_of<double>(c, 0);
-        LK(ACM_K_OTHER, Ops<double>::pass(g, 0, P_INV_SCALE, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
-        LK(ACM_K_OTHER, Ops<double>::pass(g, 1, P_INV, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
-        LK(ACM_K_OTHER, Ops<double>::x_c2r(g, 1, 1, w.st0, g.S, tgt, g.V, w.tw, c->st));
-      } else {
-        const Sym<float> sym = sym_of<float>(c, 0);
-        LK(ACM_K_OTHER, Ops<float>::pass(g, 0, P_INV_SCALE, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
-        LK(ACM_K_OTHER, Ops<float>::pass(g, 1, P_INV, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
-        LK(ACM_K_OTHER, Ops<float>::x_c2r(g, 1, 1, w.st0, g.S, tgt, g.V, w.tw, c->st));
-      }
-      if (!dev) CK(cudaMemcpyAsync(dst, w.aux, g.V * rs, cudaMemcpyDeviceToHost, c->st));
-    }
-  }
-  CK(cudaStreamSynchronize(c->st));
-  return ACM_OK;
+  return fp64 ? fft_run<double>(c, nbatch, in, out, forward) : fft_run<float>(c, nbatch, in, out, forward);
 }
 
 acm_status acm_fft_r2c(acm_ctx* c, int fp64, int nbatch, const void* in, void* out) {

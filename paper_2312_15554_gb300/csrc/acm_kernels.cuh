@@ -678,6 +678,47 @@ __global__ void __launch_bounds__(NC * 64) k_x_r2c(cx<T>* __restrict__ spec, con
   x_post_store_spec<T, N2, NC>(sm, spec + p * specProbStride, g.S, g.P, line0, tw);
 }
 
+// Line-resident R2C of one field (the bare transform): a warp owns LPW lines, whose
+// voxel pairs a lane loads as vectors and transforms from registers. `in` is aligned
+// to a pair. (k_x_r2c, two passes through shared memory per line and 128 small blocks
+// at 64^3: 10 us a launch.)
+template <typename T, int N2>
+__global__ void __launch_bounds__(XS_WARPS * 32) k_x_r2c_lr(cx<T>* __restrict__ spec, const T* __restrict__ in, Geo g,
+                                                           const cx<T>* __restrict__ twg, int gpw) {
+  using L = XL<T, N2>;
+  constexpr int M = L::M, E = L::E, TL = L::TL, LPW = L::LPW;
+  constexpr int LB = L::template lb<1>();
+  using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cx<T>* tw = reinterpret_cast<cx<T>*>(smem_raw);
+  cx<T>* lines = tw + xs_tw_slots<T, N2>();
+  xl_load_tw<T, N2, TW_MAX>(tw, twg);
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int ll = lane / TL, t = lane % TL;
+  cx<T>* bl = lines + (warp * LPW + ll) * LB;
+  const int ngroups = g.n0 * g.n1 / LPW;
+  const int gbase = (blockIdx.x * (blockDim.x >> 5) + warp) * gpw;
+#pragma unroll 1
+  for (int gi = 0; gi < gpw; ++gi) {
+    const int grp = gbase + gi;
+    if (grp >= ngroups) break;
+    const long long line = (long long)grp * LPW + ll;
+    const T* row = in + line * N2;
+    cx<T> v[E], xn;
+#pragma unroll
+    for (int m = 0; m < E; ++m) {
+      const T2 q = *reinterpret_cast<const T2*>(row + 2 * (t + TL * m));
+      v[m] = mk<T>(q.x, q.y);
+    }
+    xl_forward<T, N2>(bl, tw, t, xl_mask(), v, v, xn);
+    cx<T>* dst = spec + line * g.P;
+#pragma unroll
+    for (int m = 0; m < E; ++m) dst[t + TL * m] = v[m];
+    if (t == 0) dst[M] = xn;
+  }
+}
+
 // Line-resident C2R along the contiguous axis (acm_xline.cuh): a warp owns
 // LPW lines of one component at a time; the row arrives by cp.async, the
 // inverse transform leaves the voxel pairs 2k, 2k+1 (k = t + TL m) of the lane

@@ -37,6 +37,16 @@ struct Ops {
                            const void* in, long long inProbStride, const void* tw, cudaStream_t s);
   static cudaError_t x_c2r(const Geo& g, int nprob, int nc, const void* spec, long long specProbStride,
                            void* out, long long outProbStride, const void* tw, cudaStream_t s);
+  // the transform of one field along the contiguous axis, `in` aligned to a pair of reals
+  static cudaError_t x_r2c_lr(const Geo& g, void* spec, const void* in, const void* tw, cudaStream_t s);
+  // one field's transform along axis 0, from rows of srcPitch complex elements to rows
+  // of dstPitch; the inverse divides by V
+  static cudaError_t fft_z(const Geo& g, bool inverse, const void* src, long long srcPitch, void* dst,
+                           long long dstPitch, const void* tw, cudaStream_t s);
+  // cells of one plane: y forward, z Stokes and y inverse as one pass (where plane_pass >= 0)
+  static int plane_pass(const Geo& g);
+  static cudaError_t plane_stokes(const Geo& g, int nprob, void* spec, long long probStride, const Sym<T>& sym,
+                                  const void* tw, void* st0, void* st1, StokesDev* sprm, double* part, cudaStream_t s);
   // complex FFT pass along axis 1 (y) or 0 (z) of nc components, with operator op
   // (P_STOKES and P_SOLUTE only along z)
   static cudaError_t pass(const Geo& g, int axis, int op, int nc, int nprob, void* spec, long long probStride,

@@ -50,6 +50,18 @@ static cudaError_t set_smem(K* k, int bytes) {
     default: return cudaErrorInvalidValue;    \
   }
 
+#define ACM_DISPATCH_NI(n, FN)   \
+  switch (n) {                   \
+    case 8: return FN<T, 8>();     \
+    case 16: return FN<T, 16>();   \
+    case 32: return FN<T, 32>();   \
+    case 64: return FN<T, 64>();   \
+    case 128: return FN<T, 128>(); \
+    case 256: return FN<T, 256>(); \
+    case 512: return FN<T, 512>(); \
+    default: return 1;             \
+  }
+
 template <typename T, int N2>
 static cudaError_t l_x_local(const Geo& g, int nprob, void* spec, void* u, void* lam, const uint8_t* H,
                              const uint32_t* Hb, StokesDev* prm, double* part, const void* tw, cudaStream_t s) {
@@ -117,6 +129,17 @@ static cudaError_t l_x_r2c(const Geo& g, int nprob, int nc, void* spec, long lon
   if (nc == 1) return l_x_r2c_nc<T, N2, 1>(g, nprob, spec, sps, in, ips, tw, s);
   if (nc == 3) return l_x_r2c_nc<T, N2, 3>(g, nprob, spec, sps, in, ips, tw, s);
   return cudaErrorInvalidValue;
+}
+
+template <typename T, int N2>
+static cudaError_t l_x_r2c_lr(const Geo& g, void* spec, const void* in, const void* tw, cudaStream_t s) {
+  constexpr int smem = xs_smem_bytes<T, N2, 1, 0>();
+  static const cudaError_t attr = set_smem(k_x_r2c_lr<T, N2>, smem);
+  if (attr != cudaSuccess) return attr;
+  const XGrid x = xs_grid(g.n0 * g.n1 / XL<T, N2>::LPW);
+  k_x_r2c_lr<T, N2><<<x.blocks, x.warps * 32, xs_smem_bytes<T, N2, 1, 0>(x.warps), s>>>((cx<T>*)spec, (const T*)in, g,
+                                                                                        (const cx<T>*)tw, x.gpw);
+  return cudaGetLastError();
 }
 
 template <typename T, int N2, int NC>
@@ -254,15 +277,18 @@ static PassArgs<T> pass_args(const Geo& g, int axis, void* spec, long long probS
   a.nkx = g.n2 / 2;
   a.dm = dm;
   a.nouter = axis == 1 ? g.n0 : g.n1;
+  a.src = a.dst = a.spec;
+  a.srcRow = a.dstRow = a.rowStride;
+  a.srcOuter = a.dstOuter = a.outerStride;
   return a;
 }
 
-template <typename T, int N, int OP, int W, bool SEG>
+template <typename T, int N, int OP, int W, bool SEG, bool PLANE = false>
 static cudaError_t l_pass_w(const PassArgs<T>& a, int nc, int nprob, cudaStream_t s) {
   using C = LCfg<T, N, W>;
   constexpr int smem = lp_smem<T, N, OP, W>(), threads = lp_groups(OP) * C::NT;
   constexpr auto k = [] {
-    if constexpr (OP == OP_STOKES || OP == OP_SOLUTE) return k_lpass_z<T, N, OP, W, SEG>;
+    if constexpr (OP == OP_STOKES || OP == OP_SOLUTE) return k_lpass_z<T, N, OP, W, SEG, PLANE>;
     else if constexpr (OP == OP_FWD_SOL) return k_lpass_fsol<T, N, OP, W, SEG>;
     else if constexpr (OP == OP_INV_SOL) return k_lpass_isol<T, N, OP, W, SEG>;
     else return k_lpass<T, N, OP, W, SEG>;
@@ -284,6 +310,28 @@ static cudaError_t l_pass_pick(int w, const PassArgs<T>& a, int nc, int nprob, c
     if (w < W) return l_pass_pick<T, N, OP, W / 2, SEG>(w, a, nc, nprob, s);
   return l_pass_w<T, N, OP, W, SEG>(a, nc, nprob, s);
 }
+
+// Plane cells: y forward, Eq. 13 and y inverse in one pass along axis 1. A plane has
+// at most 65 tiles of the narrowest width, so that is the one compiled. The rounding
+// follows the y passes' choices, which have to be of one kind (see plane_pass).
+template <typename T, int N>
+static cudaError_t l_plane(const PassArgs<T>& a, bool seg, int nprob, cudaStream_t s) {
+  if constexpr (N >= 8) {
+    constexpr int W = lp_wmin<T, N>();
+    if constexpr (sizeof(T) == 4 && (N == 64 || N == 128 || N == 256))
+      if (seg) return l_pass_w<T, N, OP_STOKES, W, true, true>(a, 3, nprob, s);
+    return l_pass_w<T, N, OP_STOKES, W, false, true>(a, 3, nprob, s);
+  }
+  return cudaErrorInvalidValue;
+}
+template <typename T, int N>
+static cudaError_t l_fft_z(const PassArgs<T>& a, const Geo& g, bool inverse, cudaStream_t s) {
+  const int w = lp_width<T, N>(g, 0, OP_FWD, 0);
+  return inverse ? l_pass_pick<T, N, OP_INV_SCALE, lp_wmax<T, N>(), false>(w, a, 1, 1, s)
+                 : l_pass_pick<T, N, OP_FWD, lp_wmax<T, N>(), false>(w, a, 1, 1, s);
+}
+template <typename T, int N>
+static int l_wmin() { return lp_wmin<T, N>(); }
 
 template <typename T, int N, int OP, int NC>
 static cudaError_t l_pass_k(const Geo& g, int axis, int nprob, void* spec, long long probStride, const Sym<T>& sym,
@@ -382,6 +430,10 @@ bool Ops<T>::tx_variant(int n, int op, int nc, int shift) {
 template <typename T>
 int Ops<T>::z_blocks(const Geo& g, int op) {
   const int nc = op == P_SOLUTE ? 2 : 3;
+  if (op == P_STOKES && plane_pass(g) >= 0) {
+    auto wmin = [&]() -> int { ACM_DISPATCH_NI(g.n1, l_wmin) };
+    return rr_tiles(g.Pu, 1, wmin()).nlive;
+  }
   auto width = [&]() -> int {
     switch (g.n0) {
       case 1: return l_pass_w<T, 1>(g, 0, op, nc);
@@ -425,6 +477,11 @@ cudaError_t Ops<T>::x_r2c(const Geo& g, int nprob, int nc, void* spec, long long
 }
 
 template <typename T>
+cudaError_t Ops<T>::x_r2c_lr(const Geo& g, void* spec, const void* in, const void* tw, cudaStream_t s) {
+  ACM_DISPATCH_N(g.n2, l_x_r2c_lr, g, spec, in, tw, s)
+}
+
+template <typename T>
 cudaError_t Ops<T>::x_c2r(const Geo& g, int nprob, int nc, const void* spec, long long sps, void* out,
                           long long ops, const void* tw, cudaStream_t s) {
   ACM_DISPATCH_N(g.n2, l_x_c2r, g, nprob, nc, spec, sps, out, ops, tw, s)
@@ -438,6 +495,38 @@ cudaError_t Ops<T>::pass(const Geo& g, int axis, int op, int nc, int nprob, void
   if ((op == P_STOKES || op == P_SOLUTE || op == P_DERIV) && axis != 0) return cudaErrorInvalidValue;
   if ((op == P_FWD_SOL || op == P_INV_SOL) && axis != 1) return cudaErrorInvalidValue;
   ACM_DISPATCH_NS(n, l_pass, g, axis, op, nc, nprob, spec, ps, sym, tw, st0, st1, sprm, cprm, part, s, dm)
+}
+
+// codes of the y passes a plane pass stands for: both left to the grid or tuned to
+// row segments (-1: mixed, the three passes run in turn)
+template <typename T>
+int Ops<T>::plane_pass(const Geo& g) {
+  if (g.n0 != 1) return -1;
+  const auto& t = g.txs[sizeof(T) == 8];
+  const bool f = t[1][P_FWD] >= 3, i = t[1][P_INV] >= 3;
+  return f != i ? -1 : f;
+}
+
+template <typename T>
+cudaError_t Ops<T>::plane_stokes(const Geo& g, int nprob, void* spec, long long ps, const Sym<T>& sym, const void* tw,
+                                 void* st0, void* st1, StokesDev* sprm, double* part, cudaStream_t s) {
+  const int seg = plane_pass(g);
+  if (seg < 0) return cudaErrorInvalidValue;
+  const PassArgs<T> a = pass_args<T>(g, 1, spec, ps, sym, tw, st0, st1, sprm, nullptr, part, 0);
+  ACM_DISPATCH_N(g.n1, l_plane, a, seg == 1, nprob, s)
+}
+
+template <typename T>
+cudaError_t Ops<T>::fft_z(const Geo& g, bool inverse, const void* src, long long srcPitch, void* dst,
+                          long long dstPitch, const void* tw, cudaStream_t s) {
+  PassArgs<T> a = pass_args<T>(g, 0, dst, g.S, Sym<T>{}, tw, nullptr, nullptr, nullptr, nullptr, nullptr, 0);
+  a.src = (const cx<T>*)src;
+  a.dst = (cx<T>*)dst;
+  a.srcRow = g.n1 * srcPitch;
+  a.srcOuter = srcPitch;
+  a.dstRow = g.n1 * dstPitch;
+  a.dstOuter = dstPitch;
+  ACM_DISPATCH_NS(g.n0, l_fft_z, a, g, inverse, s)
 }
 
 template <typename T>

@@ -53,6 +53,11 @@ template <typename T>
 struct PassArgs {
   cx<T>* spec;
   long long probStride, compStride, rowStride, outerStride;
+  // plain passes: where the lines come from and go to (spec and its strides unless
+  // the caller's own array takes the place of one of them)
+  const cx<T>* src;
+  cx<T>* dst;
+  long long srcRow, srcOuter, dstRow, dstOuter;
   int Pu;           // used kx columns
   Sym<T> sym;
   const cx<T>* twg; // W_TW_MAX^k
@@ -303,11 +308,9 @@ __global__ void __launch_bounds__(LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP, W>(
   int outer, kx;
   rr_tile_lane(tl, blockIdx.x, W, col, a.Pu, &outer, &kx);
   const bool ok = kx < a.Pu;
-  cx<T>* base = a.spec + p * a.probStride + blockIdx.y * a.compStride + (long long)outer * a.outerStride + kx +
-                t * a.rowStride;
-  const long long step = TL * a.rowStride;
+  const long long field = p * a.probStride + blockIdx.y * a.compStride + kx;
   cx<T> v[E];
-  lp_load(v, base, step, ok);
+  lp_load(v, a.src + field + outer * a.srcOuter + t * a.srcRow, TL * a.srcRow, ok);
   if constexpr (OP == OP_FWD) {
     lp_fft<T, N, W, -1, SEG ? 1 : 0>(v, b, a.twg, t);
   } else {
@@ -329,7 +332,7 @@ __global__ void __launch_bounds__(LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP, W>(
     }
     lp_inverse<T, N, W, SEG>(v, b, a.twg, t);
   }
-  lp_store(v, base, step, ok);
+  lp_store(v, a.dst + field + outer * a.dstOuter + t * a.dstRow, TL * a.dstRow, ok);
 }
 
 // The y forward pass of the solute iteration, two groups of threads a block. Of
@@ -440,8 +443,11 @@ __global__ void __launch_bounds__(LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP, W>(
 // thread. Against one thread per line holding two components at a time (166
 // registers, 12 warps an SM) z Stokes takes 544 us for 606, z solute 327 for 338
 // in the block-wide tile it used; 512^3 lines, block-wide before, 5.56 ms for 6.56.
-// Blocks (tile, problem).
-template <typename T, int N, int OP, int W, bool SEG>
+//
+// PLANE: lines along axis 1 of a cell of one plane (n0 = 1, kz = 0). Axis 0 has no
+// transform there, so this is the whole of y forward, Green step and y inverse: three
+// launches of 5 to 6 us at 128 x 128 become one. Blocks (tile, problem).
+template <typename T, int N, int OP, int W, bool SEG, bool PLANE>
 __global__ void __launch_bounds__(lp_groups(OP) * LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP, W>()))
     k_lpass_z(PassArgs<T> a) {
   using C = LCfg<T, N, W>;
@@ -492,18 +498,21 @@ __global__ void __launch_bounds__(lp_groups(OP) * LCfg<T, N, W>::NT, (lp_minbloc
   }
   __syncthreads();
   const T invV = opar[4];
-  const int ky = outer;
-  const T d1 = a.sym.d1[ky], l1 = a.sym.l1[ky];
   const T d2 = ok ? a.sym.d2[kx] : (T)0, l2 = ok ? a.sym.l2[kx] : (T)0;
   const T wgt = (kx == 0 || kx == a.nkx) ? (T)1 : (T)2;
-  const T l12 = l1 + l2, d12 = sum2<false>(d1, d1, d2, d2);
+  // symbols of the other strided axis (read once: the stores below may alias them)
+  const T db = PLANE ? a.sym.d0[0] : a.sym.d1[outer], lb = PLANE ? a.sym.l0[0] : a.sym.l1[outer];
+  const T lb2 = lb + l2, db2 = sum2<false>(db, db, d2, d2);
   T acc[3] = {(T)0, (T)0, (T)0};
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const int e = grp + NC * k;
     if (e >= E) break;
-    const int kz = t + TL * e;
-    const T d0 = a.sym.d0[kz], l0 = a.sym.l0[kz];
+    const int row = t + TL * e, kz = PLANE ? 0 : row, ky = PLANE ? row : outer;
+    // the symbols of the line's axis, per element, beside the block's own
+    const T dline = PLANE ? a.sym.d1[row] : a.sym.d0[row], lr = PLANE ? a.sym.l1[row] : a.sym.l0[row];
+    const T d0 = PLANE ? db : dline, l0 = PLANE ? lb : lr, d1 = PLANE ? dline : db, l1 = PLANE ? lr : lb;
+    const T l12 = PLANE ? l1 + l2 : lb2, d12 = PLANE ? sum2<false>(d1, d1, d2, d2) : db2;
     const T L = l0 + l12, dd = d0 * d0 + d12;
     const bool k0 = (kz == 0 && ky == 0 && kx == 0);
     cx<T>* s0 = slot + e * NT;

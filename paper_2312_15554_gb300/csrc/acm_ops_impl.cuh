@@ -240,7 +240,7 @@ static int lp_width(const Geo& g, int axis, int op, int reported) {
   const int sh = g.txs[sizeof(T) == 8][axis][op];
   int w = hi;
   if (sh == 0) {
-    if ((op == OP_STOKES || op == OP_SOLUTE) && w > lo) w /= 2;
+    if ((op == OP_STOKES || op == OP_SOLUTE) && w > lo && w > rr_wdef<T>() / 2) w /= 2;
     const int nouter = axis == 1 ? g.n0 : g.n1;
     while (w > lo && rr_tiles(g.Pu, nouter, w).nlive < 304) w /= 2;
     return w;

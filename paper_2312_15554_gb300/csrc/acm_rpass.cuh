@@ -73,12 +73,13 @@ struct PassArgs {
   int nouter;       // pencils along the other strided axis
 };
 
-// values per thread: 16 in FP32; FP64 lines take smaller shares where two stages
-// allow it, for twice the warps on the two-lane FP64 pipe
+// values per thread: 16 in FP32; short FP64 lines take smaller shares, for more warps
+// on the two-lane FP64 pipes (a 32^3 z Stokes pass, 68 tiles of three warps at eight
+// values and 136 of half the columns at four: 22 us a launch and 17)
 template <typename T>
 __host__ __device__ constexpr int lp_ept(int N) {
   if (sizeof(T) == 4) return ept(N);
-  return N >= 512 ? 8 : (N >= 128 ? 16 : (N >= 32 ? 8 : (N >= 8 ? 4 : N)));
+  return N >= 512 ? 8 : (N >= 128 ? 16 : (N >= 64 ? 8 : (N >= 8 ? 4 : N)));
 }
 
 template <typename T, int N, int W>

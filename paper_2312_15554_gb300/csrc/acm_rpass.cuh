@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP, W>(
 // The y forward pass of the solute iteration, two groups of threads a block. Of
 // three blocks two take tau_1 and s' of one tile each, one per group, and one takes
 // two tiles of tau_0, which stands alone. (All three lines in one block held tau_0 at
-// the others' barriers: 237 us a launch at 256^3 and three problems, now 221.)
+// the others' barriers: 237 us a launch at 256^3 and three problems, now 215.)
 // Blocks (job, problem).
 template <typename T, int N, int OP, int W, bool SEG>
 __global__ void __launch_bounds__(2 * LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP, W>())) k_lpass_fsol(PassArgs<T> a) {
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(2 * LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP,
 // barrier between lines, and the two blocks that read b run side by side (the second
 // read hits L2). Blocks (3 tile + line, problem). At 256^3 and three problems, us a
 // launch: three lines in one thread's turn 220, two groups sharing b 229 to 243, b
-// parked in shared memory 282.
+// parked in shared memory 282; this 205.
 template <typename T, int N, int OP, int W, bool SEG>
 __global__ void __launch_bounds__(LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP, W>())) k_lpass_isol(PassArgs<T> a) {
   using C = LCfg<T, N, W>;

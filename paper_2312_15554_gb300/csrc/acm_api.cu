@@ -610,6 +610,7 @@ acm_status graph_loop_run(GraphCache& cache, const GraphKey& key, std::vector<ac
 template <typename T>
 acm_status stokes_graph_run(std::vector<StokesGroup>& grp, int deriv, bool adaptive, unsigned cap, GraphCache& cache,
                             cudaStream_t st) {
+  if (grp.size() > (size_t)LOOP_GROUPS) return ACM_ERR_ARG;  // see batch_stokes_run
   GraphKey key;
   key.prec = (int)sizeof(T);
   key.nprob = 0;
@@ -1249,7 +1250,8 @@ acm_status batch_stokes_run(acm_batch* b, const uint8_t* const* H, const acm_sto
   }
   bool prof = false;
   for (auto& gr : b->groups) prof = prof || gr.c->prof;
-  if (P.device_loop && !prof) {
+  // one loop node watches at most LOOP_GROUPS shapes
+  if (P.device_loop && !prof && grp.size() <= (size_t)LOOP_GROUPS) {
     CKS(stokes_graph_run<T>(grp, P.deriv, P.adaptive != 0, (unsigned)P.max_iter, b->graph, b->st));
   } else {
     for (auto& x : grp)

@@ -83,11 +83,14 @@ cudaError_t count_faces_add(const uint8_t* H, int n0, int n1, int n2, unsigned l
 // Condition of the device-resident loop (a CUDA graph while node): continue
 // while any problem of any group has not set its stop flag, and at most `cap`
 // iterations. Group g has n[g] control blocks of `stride` bytes starting at
-// base[g]; the stop flag is the int at byte offset `done_off` of each block.
+// base[g]; the stop flag is the int at byte offset `done_off` of each block. The
+// groups are a kernel argument, at most LOOP_GROUPS of them; work with more runs in
+// the host-launched loop.
+constexpr int LOOP_GROUPS = 16;
 struct LoopCtl {
-  const char* base[4];
-  int n[4];
-  int stride[4];
+  const char* base[LOOP_GROUPS];
+  int n[LOOP_GROUPS];
+  int stride[LOOP_GROUPS];
   int ngroups;
   int done_off;
   unsigned int* counter;  // iterations run so far (device)

@@ -76,13 +76,14 @@ __device__ __forceinline__ void load_tw_x(cx<T>* tw, const cx<T>* __restrict__ t
 // is loaded once and written once.
 template <typename T, int N2, int NC>
 __device__ __forceinline__ void x_load_spec_pre(cx<T>* sm, const cx<T>* __restrict__ spec, long long S, int P,
-                                                int line0, const cx<T>* twx) {
+                                                int line0, int lines, const cx<T>* twx) {
   using C = XCfg<T, N2>;
   constexpr int M = C::M;
   const cx<T>* tw = twx + tw_total(M);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int cl = warp; cl < NC * C::LPB; cl += nw) {
     const int c = cl / C::LPB, l = cl - c * C::LPB;
+    if (l >= lines) continue;
     const cx<T>* src = spec + c * S + (long long)(line0 + l) * P;
     cx<T>* s = sm + cl * C::LS;
     for (int k = lane; k <= M / 2; k += 32) {
@@ -99,7 +100,7 @@ __device__ __forceinline__ void x_load_spec_pre(cx<T>* sm, const cx<T>* __restri
 // written to global memory.
 template <typename T, int N2, int NC>
 __device__ __forceinline__ void x_post_store_spec(const cx<T>* sm, cx<T>* __restrict__ spec, long long S, int P,
-                                                  int line0, const cx<T>* twx) {
+                                                  int line0, int lines, const cx<T>* twx) {
   using C = XCfg<T, N2>;
   constexpr int M = C::M;
   const cx<T>* tw = twx + tw_total(M);
@@ -107,6 +108,7 @@ __device__ __forceinline__ void x_post_store_spec(const cx<T>* sm, cx<T>* __rest
   const T half = (T)0.5;
   for (int cl = warp; cl < NC * C::LPB; cl += nw) {
     const int c = cl / C::LPB, l = cl - c * C::LPB;
+    if (l >= lines) continue;
     cx<T>* dst = spec + c * S + (long long)(line0 + l) * P;
     const cx<T>* s = sm + cl * C::LS;
     for (int k = lane; k <= M / 2; k += 32) {
@@ -123,6 +125,14 @@ __device__ __forceinline__ void x_post_store_spec(const cx<T>* sm, cx<T>* __rest
       }
     }
   }
+}
+
+// Lines of a block that exist: all LPB, except on planes of 32 lines with n2 <= 32,
+// whose single block holds 64. The transform runs on the empty line buffers too (each
+// line is private to its lanes), nothing is loaded into or stored from them.
+template <typename T, int N2>
+__device__ __forceinline__ int x_lines(const Geo& g, int line0) {
+  return min(XCfg<T, N2>::LPB, g.n0 * g.n1 - line0);
 }
 
 // complex FFT of length M on NC * LPB component lines, TL threads per line
@@ -665,17 +675,18 @@ __global__ void __launch_bounds__(NC * 64) k_x_r2c(cx<T>* __restrict__ spec, con
   cx<T>* tw = sm + NC * C::LPB * C::LS;
   const int p = blockIdx.y;
   const int line0 = blockIdx.x * C::LPB;
+  const int lines = x_lines<T, N2>(g, line0);
   const T* ip = in + p * inProbStride;
   load_tw_x<T, N2>(tw, twg);
   for (int idx = threadIdx.x; idx < NC * C::LPB * N2; idx += blockDim.x) {
     const int n = idx & (N2 - 1), cl = idx / N2;
     const int c = cl / C::LPB, l = cl - c * C::LPB;
-    re_at(sm + cl * C::LS, n) = ip[c * g.V + (long long)(line0 + l) * N2 + n];
+    re_at(sm + cl * C::LS, n) = l < lines ? ip[c * g.V + (long long)(line0 + l) * N2 + n] : (T)0;
   }
   __syncthreads();
   x_fft<T, N2, NC, -1>(sm, tw);
   __syncthreads();
-  x_post_store_spec<T, N2, NC>(sm, spec + p * specProbStride, g.S, g.P, line0, tw);
+  x_post_store_spec<T, N2, NC>(sm, spec + p * specProbStride, g.S, g.P, line0, lines, tw);
 }
 
 // Line-resident R2C of one field (the bare transform): a warp owns LPW lines, whose
@@ -780,17 +791,18 @@ __global__ void __launch_bounds__(NC * 64) k_x_c2r(const cx<T>* __restrict__ spe
   cx<T>* tw = sm + NC * C::LPB * C::LS;
   const int p = blockIdx.y;
   const int line0 = blockIdx.x * C::LPB;
+  const int lines = x_lines<T, N2>(g, line0);
   T* op = out + p * outProbStride;
   load_tw_x<T, N2>(tw, twg);
   __syncthreads();
-  x_load_spec_pre<T, N2, NC>(sm, spec + p * specProbStride, g.S, g.P, line0, tw);
+  x_load_spec_pre<T, N2, NC>(sm, spec + p * specProbStride, g.S, g.P, line0, lines, tw);
   __syncthreads();
   x_fft<T, N2, NC, +1>(sm, tw);
   __syncthreads();
   for (int idx = threadIdx.x; idx < NC * C::LPB * N2; idx += blockDim.x) {
     const int n = idx & (N2 - 1), cl = idx / N2;
     const int c = cl / C::LPB, l = cl - c * C::LPB;
-    op[c * g.V + (long long)(line0 + l) * N2 + n] = re_at(sm + cl * C::LS, n);
+    if (l < lines) op[c * g.V + (long long)(line0 + l) * N2 + n] = re_at(sm + cl * C::LS, n);
   }
 }
 

@@ -119,7 +119,7 @@ static cudaError_t l_x_r2c_nc(const Geo& g, int nprob, void* spec, long long sps
   constexpr int smem = x_smem_bytes<T, N2, NC>();
   static const cudaError_t attr = set_smem(k_x_r2c<T, N2, NC>, smem);
   if (attr != cudaSuccess) return attr;
-  dim3 grid(g.n0 * g.n1 / XCfg<T, N2>::LPB, nprob);
+  dim3 grid((g.n0 * g.n1 + XCfg<T, N2>::LPB - 1) / XCfg<T, N2>::LPB, nprob);
   k_x_r2c<T, N2, NC><<<grid, NC * 64, smem, s>>>((cx<T>*)spec, (const T*)in, g, ips, sps, (const cx<T>*)tw);
   return cudaGetLastError();
 }
@@ -148,7 +148,7 @@ static cudaError_t l_x_c2r_nc(const Geo& g, int nprob, const void* spec, long lo
   constexpr int smem = x_smem_bytes<T, N2, NC>();
   static const cudaError_t attr = set_smem(k_x_c2r<T, N2, NC>, smem);
   if (attr != cudaSuccess) return attr;
-  dim3 grid(g.n0 * g.n1 / XCfg<T, N2>::LPB, nprob);
+  dim3 grid((g.n0 * g.n1 + XCfg<T, N2>::LPB - 1) / XCfg<T, N2>::LPB, nprob);
   k_x_c2r<T, N2, NC><<<grid, NC * 64, smem, s>>>((const cx<T>*)spec, (T*)out, g, ops, sps, (const cx<T>*)tw);
   return cudaGetLastError();
 }

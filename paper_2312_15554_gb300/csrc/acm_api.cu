@@ -15,6 +15,7 @@
 
 #include "acm.h"
 #include "acm_ops.h"
+#include "acm_ptr.h"
 
 using namespace acm;
 
@@ -173,14 +174,15 @@ bool shape_ok(int n0, int n1, int n2) {
   return (pow2_in_range(n0) || (n0 == 1 && n1 >= 32)) && pow2_in_range(n1) && pow2_in_range(n2);
 }
 
+// whether kernels of this context may touch p; anything else, host memory and other
+// GPUs' memory alike, goes through a copy of kind cudaMemcpyDefault
 bool is_device_ptr(const void* p) {
-  if (!p) return false;
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+  int dev = 0;
+  if (!p || cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+  return on_device(p, dev);
 }
 
 // captured loops hold kernel arguments (tile widths, buffers): drop them
@@ -1492,7 +1494,7 @@ acm_status fft_run(acm_ctx* c, int nbatch, const void* in, void* out, bool forwa
     if (forward) {
       const void* x = src;
       if (!in_dev) {
-        CK(cudaMemcpyAsync(w.aux, src, g.V * rs, cudaMemcpyHostToDevice, c->st));
+        CK(cudaMemcpyAsync(w.aux, src, g.V * rs, cudaMemcpyDefault, c->st));
         x = w.aux;
       }
       if ((uintptr_t)x % cs == 0) LK(ACM_K_OTHER, Ops<T>::x_r2c_lr(g, w.st0, x, w.tw, c->st));
@@ -1507,7 +1509,7 @@ acm_status fft_run(acm_ctx* c, int nbatch, const void* in, void* out, bool forwa
       LK(ACM_K_OTHER, Ops<T>::fft_z(g, true, direct ? (const void*)src : w.st0, direct ? g.Pu : g.P, w.st0, g.P, w.tw, c->st));
       LK(ACM_K_OTHER, Ops<T>::pass(g, 1, P_INV, 1, 1, w.st0, g.S, sym, w.tw, 0, 0, 0, 0, 0, c->st));
       LK(ACM_K_OTHER, Ops<T>::x_c2r(g, 1, 1, w.st0, g.S, out_dev ? (void*)dst : w.aux, g.V, w.tw, c->st));
-      if (!out_dev) CK(cudaMemcpyAsync(dst, w.aux, g.V * rs, cudaMemcpyDeviceToHost, c->st));
+      if (!out_dev) CK(cudaMemcpyAsync(dst, w.aux, g.V * rs, cudaMemcpyDefault, c->st));
     }
   }
   CK(cudaStreamSynchronize(c->st));

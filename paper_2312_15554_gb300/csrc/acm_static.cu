@@ -20,6 +20,7 @@
 
 #include "acm.h"
 #include "acm_ops.h"
+#include "acm_ptr.h"
 
 using namespace acm;
 
@@ -90,17 +91,6 @@ acm_status setup_current_device(int dev, DeviceSetup** out) {
   }
   *out = &s;
   return ACM_OK;
-}
-
-// device memory of the current device `dev` (the kernels run there and read
-// and write the buffers directly), or managed memory
-bool on_device(const void* p, int dev) {
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
 }
 
 template <typename T>

@@ -701,10 +701,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32) k_x_r2c_lr(cx<T>* __restrict__ 
   constexpr int LB = L::template lb<1>();
   using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<T>* tw = reinterpret_cast<cx<T>*>(smem_raw);
-  cx<T>* lines = tw + xs_tw_slots<T, N2>();
-  xl_load_tw<T, N2, TW_MAX>(tw, twg);
-  __syncthreads();
+  cx<T>* lines = reinterpret_cast<cx<T>*>(smem_raw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ll = lane / TL, t = lane % TL;
   cx<T>* bl = lines + (warp * LPW + ll) * LB;
@@ -722,7 +719,7 @@ __global__ void __launch_bounds__(XS_WARPS * 32) k_x_r2c_lr(cx<T>* __restrict__ 
       const T2 q = *reinterpret_cast<const T2*>(row + 2 * (t + TL * m));
       v[m] = mk<T>(q.x, q.y);
     }
-    xl_forward<T, N2>(bl, tw, t, xl_mask(), v, v, xn);
+    xl_forward<T, N2, TW_MAX>(bl, twg, t, xl_mask(), v, v, xn);
     cx<T>* dst = spec + line * g.P;
 #pragma unroll
     for (int m = 0; m < E; ++m) dst[t + TL * m] = v[m];

@@ -115,6 +115,14 @@ __device__ __forceinline__ cx<T> xl_post(cx<T> Zk, cx<T> Zm, cx<T> wt) {
   return a - mul_i(root_mul<-1, m, 2 * E>(cmul(wt, b)));
 }
 
+// the same with W^k itself
+template <typename T>
+__device__ __forceinline__ cx<T> xl_post_tab(cx<T> Zk, cx<T> Zm, cx<T> wk) {
+  const T h = (T)0.5;
+  const cx<T> a = cscale(Zk + cconj(Zm), h), b = cscale(Zk - cconj(Zm), h);
+  return a - mul_i(cmul_fma<0>(wk, b));
+}
+
 // Second Stockham stage (radix TL, span E) between shared memory and v:
 // reads positions t + TL i + E r, writes nothing; v[i + NB r] = outputs.
 // Its twiddles W_M^{j r} (j = t + TL i) are W_M^{t r} exp(-2 pi i i r / E):
@@ -143,6 +151,28 @@ __device__ __forceinline__ void xl_stage2(const cx<T>* sl, const cx<T>* tw, int 
 #pragma unroll
     for (int r = 0; r < TL; ++r) v[i + NB * r] = w2[r];
   });
+}
+
+// The second stage of a forward transform with every twiddle read from the master
+// table W_TWM^k, each a correctly rounded root: the product of a loaded and a
+// compile-time root above is one rounding more per value.
+template <typename T, int N2, int TWM>
+__device__ __forceinline__ void xl_stage2_tab(const cx<T>* sl, const cx<T>* __restrict__ master, int t,
+                                              cx<T> (&v)[XL<T, N2>::E]) {
+  using L = XL<T, N2>;
+  constexpr int E = L::E, TL = L::TL, NB = L::NB, M = L::M;
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int j = t + TL * i;
+    cx<T> w2[TL];
+#pragma unroll
+    for (int r = 0; r < TL; ++r) w2[r] = sl[pad(j + E * r)];
+#pragma unroll
+    for (int r = 1; r < TL; ++r) w2[r] = cmul_fma<0>(w2[r], master[j * r * (TWM / M)]);
+    dft<TL, -1>(w2);
+#pragma unroll
+    for (int r = 0; r < TL; ++r) v[i + NB * r] = w2[r];
+  }
 }
 
 // Inverse real transform of one line. sl holds the half spectrum X[0..M]
@@ -181,7 +211,8 @@ __device__ __forceinline__ void xl_inverse(cx<T>* sl, const cx<T>* tw, int t, un
 // lane (TL - t) mod TL of its line) instead of a second pass through sl.
 // Positions m and E-1-m are finished together; lane 0's partner E - m of
 // position m was overwritten one step earlier and is carried in a register.
-template <typename T, int N2>
+// TWM > 0: tw is the master table W_TWM^k and every twiddle is read from it.
+template <typename T, int N2, int TWM = 0>
 __device__ __forceinline__ void xl_forward(cx<T>* sl, const cx<T>* tw, int t, unsigned mask,
                                            cx<T> (&v)[XL<T, N2>::E], cx<T> (&X)[XL<T, N2>::E], cx<T>& xn) {
   using L = XL<T, N2>;
@@ -194,9 +225,15 @@ __device__ __forceinline__ void xl_forward(cx<T>* sl, const cx<T>* tw, int t, un
   for (int r = 0; r < E; ++r) sl[pad(t * E + r)] = v[r];
   if constexpr (TL > 1) {
     __syncwarp(mask);
-    xl_stage2<T, N2, -1>(sl, tw, t, v);
+    if constexpr (TWM > 0) xl_stage2_tab<T, N2, TWM>(sl, tw, t, v);
+    else xl_stage2<T, N2, -1>(sl, tw, t, v);
     __syncwarp(mask);  // the stage-2 reads are done before sl is reused
   }
+  auto post = [&](auto P, cx<T> zk, cx<T> zp) {
+    constexpr int m = decltype(P)::value;
+    if constexpr (TWM > 0) return xl_post_tab(zk, zp, tw[(t + TL * m) * (TWM / N2)]);
+    else return xl_post<m, E>(zk, zp, wt);
+  };
   // Z_k sits in v[m] of its own lane
   const int lane = threadIdx.x & 31;
   const int src = (lane - t) + (TL - t) % TL;
@@ -218,9 +255,9 @@ __device__ __forceinline__ void xl_forward(cx<T>* sl, const cx<T>* tw, int t, un
       X[m] = mk<T>(a.x + a.y, (T)0);
       xn = mk<T>(a.x - a.y, (T)0);
     } else {
-      X[m] = xl_post<m, E>(a, zm, wt);
+      X[m] = post(ic<m>{}, a, zm);
     }
-    X[mb] = xl_post<mb, E>(b, zb, wt);
+    X[mb] = post(ic<mb>{}, b, zb);
   });
 }
 

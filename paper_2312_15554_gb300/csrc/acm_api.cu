@@ -16,6 +16,7 @@
 #include "acm.h"
 #include "acm_ops.h"
 #include "acm_ptr.h"
+#include "acm_roots.h"
 
 using namespace acm;
 
@@ -258,10 +259,14 @@ acm_status ensure_prec(acm_ctx* c) {
   CK(cudaMemset(w.st0, 0, (size_t)c->B * g.S * cs));
   CK(cudaMemset(w.st1, 0, (size_t)c->B * g.S * cs));
   std::vector<T> tw(2 * TW_MAX);
-  const double PI = 3.14159265358979323846;
-  for (int k = 0; k < TW_MAX; ++k) {
-    tw[2 * k] = (T)std::cos(2.0 * PI * k / TW_MAX);
-    tw[2 * k + 1] = (T)(-std::sin(2.0 * PI * k / TW_MAX));
+  if constexpr (sizeof(T) == 8) {
+    unit_roots(TW_MAX, tw.data());
+  } else {
+    const double PI = 3.14159265358979323846;
+    for (int k = 0; k < TW_MAX; ++k) {
+      tw[2 * k] = (T)std::cos(2.0 * PI * k / TW_MAX);
+      tw[2 * k + 1] = (T)(-std::sin(2.0 * PI * k / TW_MAX));
+    }
   }
   CK(cudaMemcpy(w.tw, tw.data(), tw.size() * sizeof(T), cudaMemcpyHostToDevice));
   std::vector<T> sym;

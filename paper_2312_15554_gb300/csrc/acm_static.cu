@@ -21,6 +21,7 @@
 #include "acm.h"
 #include "acm_ops.h"
 #include "acm_ptr.h"
+#include "acm_roots.h"
 
 using namespace acm;
 
@@ -72,12 +73,11 @@ acm_status setup_current_device(int dev, DeviceSetup** out) {
     s.tw64 = p;
     static double h64[2 * TW_MAX];
     static float h32[2 * TW_MAX];
+    unit_roots(TW_MAX, h64);
     const double PI = 3.14159265358979323846;
     for (int k = 0; k < TW_MAX; ++k) {
-      h64[2 * k] = std::cos(2.0 * PI * k / TW_MAX);
-      h64[2 * k + 1] = -std::sin(2.0 * PI * k / TW_MAX);
-      h32[2 * k] = (float)h64[2 * k];
-      h32[2 * k + 1] = (float)h64[2 * k + 1];
+      h32[2 * k] = (float)std::cos(2.0 * PI * k / TW_MAX);
+      h32[2 * k + 1] = (float)-std::sin(2.0 * PI * k / TW_MAX);
     }
     // a copy from pageable memory may return before its DMA lands; the device
     // synchronisation orders the tables before work on any (non-blocking) stream

@@ -39,8 +39,12 @@ struct XL {
   static constexpr int LPW = 32 / TL;     // lines per warp
   static constexpr int NB = E / TL;       // second-stage groups per lane (TL > 1)
   static_assert(TL <= E && E * TL == M, "two stages: radix E, then radix TL");
-  // twiddle table of a block: W_N2^t (t < TL), then W_M^{t r} at TL r + t (r = 1..TL-1)
-  static constexpr int TW = TL * TL;
+  // twiddle table of a block: W_N2^t (t < TL), then W_M^{t r} at TL r + t (r = 1..TL-1);
+  // in FP64 also W_N2^k (k < M): the product of W^t and a compile-time root would cost
+  // the FP64 pipe another multiplication, and each value another rounding (shorter
+  // shares a lane than FP32's have more values with t > 0)
+  static constexpr bool TAB = sizeof(T) == 8;
+  static constexpr int TW0 = TL * TL, TW = TW0 + (TAB ? M : 0);
   // slots per line buffer: X[0..M] (pad(M) included), bank-friendly for TL lanes
   static constexpr int LS = line_stride(M + 1, TL, 0, wave_slots<T>());
   // stride between the consecutive lines of a warp holding NBUF buffers each:
@@ -62,7 +66,8 @@ __device__ __forceinline__ void xl_load_tw(cx<T>* tw, const cx<T>* __restrict__ 
   using L = XL<T, N2>;
   for (int e = threadIdx.x; e < L::TW; e += blockDim.x) {
     const int r = e / L::TL, t = e - r * L::TL;
-    tw[e] = master[r == 0 ? t * (TWM / N2) : ((t * r) % L::M) * (TWM / L::M)];
+    if (L::TAB && e >= L::TW0) tw[e] = master[(e - L::TW0) * (TWM / N2)];
+    else tw[e] = master[r == 0 ? t * (TWM / N2) : ((t * r) % L::M) * (TWM / L::M)];
   }
 }
 
@@ -121,6 +126,12 @@ __device__ __forceinline__ cx<T> xl_post_tab(cx<T> Zk, cx<T> Zm, cx<T> wk) {
   const T h = (T)0.5;
   const cx<T> a = cscale(Zk + cconj(Zm), h), b = cscale(Zk - cconj(Zm), h);
   return a - mul_i(cmul_fma<0>(wk, b));
+}
+
+template <typename T>
+__device__ __forceinline__ cx<T> xl_pre_tab(cx<T> X, cx<T> Y, cx<T> wk) {
+  const cx<T> e = X + cconj(Y), o = cmul(X - cconj(Y), cconj(wk));
+  return e + mul_i(o);
 }
 
 // Second Stockham stage (radix TL, span E) between shared memory and v:
@@ -187,7 +198,8 @@ __device__ __forceinline__ void xl_inverse(cx<T>* sl, const cx<T>* tw, int t, un
   static_for<E>([&](auto R) {
     constexpr int r = decltype(R)::value;
     const int k = t + TL * r;
-    v[r] = xl_pre<r, E>(sl[pad(k)], sl[pad(M - k)], wt);
+    if constexpr (L::TAB) v[r] = xl_pre_tab(sl[pad(k)], sl[pad(M - k)], tw[L::TW0 + k]);
+    else v[r] = xl_pre<r, E>(sl[pad(k)], sl[pad(M - k)], wt);
   });
   dft<E, +1>(v);
   if constexpr (TL > 1) {
@@ -232,6 +244,7 @@ __device__ __forceinline__ void xl_forward(cx<T>* sl, const cx<T>* tw, int t, un
   auto post = [&](auto P, cx<T> zk, cx<T> zp) {
     constexpr int m = decltype(P)::value;
     if constexpr (TWM > 0) return xl_post_tab(zk, zp, tw[(t + TL * m) * (TWM / N2)]);
+    else if constexpr (L::TAB) return xl_post_tab(zk, zp, tw[L::TW0 + t + TL * m]);
     else return xl_post<m, E>(zk, zp, wt);
   };
   // Z_k sits in v[m] of its own lane

@@ -256,7 +256,8 @@ acm_status acm_batch_stokes(acm_batch* batch, const uint8_t* const* H, const acm
  * y-inverse solute (0 where a pass does not apply). At 64, 128 and 256 points the
  * tuner's candidates are row segments of 128 and 64 bytes, reported as negative
  * widths (FP32 -16 and -8, FP64 -8 and -4), except in the z solute pass; in FP32 they
- * round differently from the positive widths (about 1e-7 of a field).
+ * round differently from the positive widths (about 1e-7 of a field). FP32 passes of
+ * 128 and 256 points also offer -4, tried where a pass left alone takes 4 columns.
  * acm_set_tiles sets widths explicitly (ACM_ERR_ARG for one outside the set that
  * the pass offers); a pass runs the nearest width that is compiled for its line
  * length, and the default width leaves the choice to the grid. acm_get_tiles reads

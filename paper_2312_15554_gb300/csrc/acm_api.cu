@@ -1361,15 +1361,20 @@ acm_status autotune_ctx(acm_ctx* c, int nprob, int deriv) {
     const int n = j.axis == 1 ? c->g.n1 : c->g.n0;
     float best = 0;
     int best_sh = 0;
-    // Where the row-segment widths (3, 4) exist they are the candidates, except for
+    // Where the row-segment widths (3 to 5) exist they are the candidates, except for
     // the solute z pass, which takes the others: the choices of either set agree bit
-    // for bit, so a tuned context's results do not hang on which of them won.
+    // for bit, so a tuned context's results do not hang on which of them won. The
+    // narrowest is timed on the grids that would run it untuned.
     const bool seg = Ops<T>::tx_variant(n, j.op, j.nc, 3);
-    const int first = seg && j.op != P_SOLUTE ? 3 : -1, last = seg && j.op == P_SOLUTE ? 2 : 4;
+    const int first = seg && j.op != P_SOLUTE ? 3 : -1, last = seg && j.op == P_SOLUTE ? 2 : MAX_TILE_CHOICE;
+    Geo gd = c->g;
+    gd.txs[pr][j.axis][j.op] = 0;
+    const int untuned = Ops<T>::pass_columns(gd, j.axis, j.op, j.nc);
     for (int sh = first; sh <= last && st == ACM_OK; ++sh) {
       if (!Ops<T>::tx_variant(n, j.op, j.nc, sh)) continue;
       Geo g = c->g;
       g.txs[pr][j.axis][j.op] = (signed char)sh;
+      if (sh == 5 && Ops<T>::pass_columns(g, j.axis, j.op, j.nc) < untuned) continue;
       const long long ps = (j.solute ? 4LL : 3LL) * g.S;
       StokesDev* sp = j.solute ? nullptr : c->sprm;
       SoluteDev* cp = j.solute ? c->cprm : nullptr;
@@ -1444,7 +1449,7 @@ acm_status ctx_create(acm_ctx** out, int n0, int n1, int n2, void* stream, int B
   const int nbx = std::max(Ops<float>::x_blocks(g), Ops<double>::x_blocks(g));
   // partial sums sized for the narrowest tile any choice may give
   int nbz = 0;
-  for (int sh = -1; sh <= 4; ++sh) {
+  for (int sh = -1; sh <= MAX_TILE_CHOICE; ++sh) {
     Geo gn = g;
     for (int pr = 0; pr < 2; ++pr)
       for (int op : {P_STOKES, P_SOLUTE}) gn.txs[pr][0][op] = (signed char)sh;
@@ -1808,7 +1813,7 @@ acm_status acm_set_tiles(acm_ctx* c, int fp64, const int tiles[NTUNE]) {
     if (j.solute && c->spec_comps < 4) continue;
     const int n = j.axis == 1 ? g.n1 : g.n0;
     bool found = false;
-    for (int sh = -1; sh <= 4 && !found; ++sh) {
+    for (int sh = -1; sh <= MAX_TILE_CHOICE && !found; ++sh) {
       if (!(fp64 ? Ops<double>::tx_variant(n, j.op, j.nc, sh) : Ops<float>::tx_variant(n, j.op, j.nc, sh))) continue;
       g.txs[fp64][j.axis][j.op] = (signed char)sh;
       const int tx = fp64 ? Ops<double>::pass_tx(g, j.axis, j.op, j.nc) : Ops<float>::pass_tx(g, j.axis, j.op, j.nc);

@@ -18,9 +18,10 @@ struct Ops {
   // blocks per problem of the x-passes and of a z-pass (number of partial sums)
   static int x_blocks(const Geo& g);
   static int z_blocks(const Geo& g, int op);
-  // tile width (columns) a strided pass reports under g's tile choice, and
-  // whether the choice `shift` (-1 .. 4) is one of its own
+  // tile width (columns) a strided pass reports under g's tile choice and the one it
+  // runs with, and whether the choice `shift` (-1 .. MAX_TILE_CHOICE) is one of its own
   static int pass_tx(const Geo& g, int axis, int op, int nc);
+  static int pass_columns(const Geo& g, int axis, int op, int nc);
   static bool tx_variant(int n, int op, int nc, int shift);
 
   static cudaError_t x_stokes_local(const Geo& g, int nprob, void* spec, void* u, void* lam,

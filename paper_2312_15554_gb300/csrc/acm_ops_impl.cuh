@@ -176,7 +176,11 @@ static cudaError_t l_x_c2r(const Geo& g, int nprob, int nc, const void* spec, lo
 // grid; the solver passes at N >= 64 also take -1, 1, 2 (half, double, four
 // times the default width reported, where that number stays within 2..32 columns,
 // 1536 line threads and 200 KB) and, at N = 64, 128 and 256, 3 and 4 (a full and
-// a half 128-byte row segment, reported as -W).
+// a half 128-byte row segment, reported as -W). FP32 lines of 128 and 256 points also
+// take 5, a quarter segment: what a pass of a small grid picks by itself, so the tuner
+// has to be able to pick it too (z Stokes, us a launch at half and quarter segments:
+// 22.4 and 17.0 at 256 x 32 x 64, 15.3 and 13.5 at 128 x 64 x 32; y at 16 x 256 x 64
+// 10.3 and 8.4).
 template <int N, int OP, int NC>
 constexpr bool tunable() {
   return N >= 64 && ((OP == OP_FWD && NC == 3) || (OP == OP_INV && NC == 3) || OP == OP_STOKES || OP == OP_SOLUTE ||
@@ -198,6 +202,10 @@ constexpr bool rr_ok() {
 template <typename T>
 constexpr int rr_wdef() { return 128 / (int)sizeof(cx<T>); }
 
+// whether lines of N are compiled for a quarter of that
+template <typename T, int N>
+constexpr bool rr_quarter() { return sizeof(T) == 4 && (N == 128 || N == 256); }
+
 // the width (T, N, OP, NC) reports under the choice `shift`
 template <typename T, int N, int OP, int NC>
 constexpr int resolved_tx(int shift) {
@@ -205,6 +213,7 @@ constexpr int resolved_tx(int shift) {
   if constexpr (rr_ok<T, N, OP, NC>()) {
     if (shift == 3) return -rr_wdef<T>();
     if (shift == 4) return -rr_wdef<T>() / 2;
+    if (shift == 5 && rr_quarter<T, N>()) return -rr_wdef<T>() / 4;
   }
   if (tunable<N, OP, NC>()) {
     if (shift < 0 && tx_ok<T, N, OP, NC, TX0 / 2>()) return TX0 / 2;
@@ -222,6 +231,7 @@ constexpr int lp_wmin() {
   constexpr int TL = N / lp_ept<T>(N);
   return TL >= 8 ? 4 : 32 / TL;
 }
+static_assert(lp_wmin<float, 128>() == rr_wdef<float>() / 4 && lp_wmin<float, 256>() == rr_wdef<float>() / 4);
 template <typename T, int N>
 constexpr int lp_wmax() {
   constexpr int m = N == 512 ? rr_wdef<T>() / 2 : rr_wdef<T>();
@@ -428,26 +438,27 @@ bool Ops<T>::tx_variant(int n, int op, int nc, int shift) {
 }
 
 template <typename T>
+int Ops<T>::pass_columns(const Geo& g, int axis, int op, int nc) {
+  switch (axis == 1 ? g.n1 : g.n0) {
+    case 1: return l_pass_w<T, 1>(g, axis, op, nc);
+    case 8: return l_pass_w<T, 8>(g, axis, op, nc);
+    case 16: return l_pass_w<T, 16>(g, axis, op, nc);
+    case 32: return l_pass_w<T, 32>(g, axis, op, nc);
+    case 64: return l_pass_w<T, 64>(g, axis, op, nc);
+    case 128: return l_pass_w<T, 128>(g, axis, op, nc);
+    case 256: return l_pass_w<T, 256>(g, axis, op, nc);
+    case 512: return l_pass_w<T, 512>(g, axis, op, nc);
+    default: return 1;
+  }
+}
+
+template <typename T>
 int Ops<T>::z_blocks(const Geo& g, int op) {
-  const int nc = op == P_SOLUTE ? 2 : 3;
   if (op == P_STOKES && plane_pass(g) >= 0) {
     auto wmin = [&]() -> int { ACM_DISPATCH_NI(g.n1, l_wmin) };
     return rr_tiles(g.Pu, 1, wmin()).nlive;
   }
-  auto width = [&]() -> int {
-    switch (g.n0) {
-      case 1: return l_pass_w<T, 1>(g, 0, op, nc);
-      case 8: return l_pass_w<T, 8>(g, 0, op, nc);
-      case 16: return l_pass_w<T, 16>(g, 0, op, nc);
-      case 32: return l_pass_w<T, 32>(g, 0, op, nc);
-      case 64: return l_pass_w<T, 64>(g, 0, op, nc);
-      case 128: return l_pass_w<T, 128>(g, 0, op, nc);
-      case 256: return l_pass_w<T, 256>(g, 0, op, nc);
-      case 512: return l_pass_w<T, 512>(g, 0, op, nc);
-      default: return 1;
-    }
-  };
-  return rr_tiles(g.Pu, g.n1, width()).nlive;
+  return rr_tiles(g.Pu, g.n1, pass_columns(g, 0, op, op == P_SOLUTE ? 2 : 3)).nlive;
 }
 
 template <typename T>

@@ -58,6 +58,8 @@ enum { ST_OK = 0, ST_MAXITER = -4, ST_DIVERGED = -5, ST_NONFINITE = -6 };
 // that problem in FP64; never returned to the caller)
 enum { ST_STALLED = -100 };
 
+constexpr int MAX_TILE_CHOICE = 5;  // the choices of Geo::txs are -1 .. 5
+
 // Geometry of one grid and its half spectrum.
 struct Geo {
   int n0, n1, n2;
@@ -69,8 +71,8 @@ struct Geo {
   long long us; // stride of the advecting velocity between problems (0: shared)
   int lph;      // problems per indicator: problem p uses H + (p / lph) * hs
   // tile-width choice of the strided passes per [precision (FP64 = 1)][axis][pass op]:
-  // 0 by the grid; -1 half, +1 double, +2 four times the default width; +3, +4 row
-  // segments of 128 and 64 bytes (set by the autotuner)
+  // 0 by the grid; -1 half, +1 double, +2 four times the default width; +3, +4, +5
+  // row segments of 128, 64 and 32 bytes (set by the autotuner)
   signed char txs[2][2][8] = {};
 };
 

@@ -690,9 +690,14 @@ __global__ void __launch_bounds__(NC * 64) k_x_r2c(cx<T>* __restrict__ spec, con
 }
 
 // Line-resident R2C of one field (the bare transform): a warp owns LPW lines, whose
-// voxel pairs a lane loads as vectors and transforms from registers. `in` is aligned
-// to a pair. (k_x_r2c, two passes through shared memory per line and 128 small blocks
+// voxel pairs a lane loads as vectors and transforms from registers, with tabulated
+// twiddles: FP32 results are those of k_x_r2c bit for bit. `in` is aligned to a pair. (k_x_r2c, two passes through shared memory per line and 128 small blocks
 // at 64^3: 10 us a launch.)
+template <typename T, int N2>
+__host__ __device__ constexpr int xr_smem_bytes(int warps = XS_WARPS) {
+  return (N2 + warps * XL<T, N2>::LPW * XL<T, N2>::template lb<1>()) * (int)sizeof(cx<T>);
+}
+
 template <typename T, int N2>
 __global__ void __launch_bounds__(XS_WARPS * 32) k_x_r2c_lr(cx<T>* __restrict__ spec, const T* __restrict__ in, Geo g,
                                                            const cx<T>* __restrict__ twg, int gpw) {
@@ -701,25 +706,32 @@ __global__ void __launch_bounds__(XS_WARPS * 32) k_x_r2c_lr(cx<T>* __restrict__ 
   constexpr int LB = L::template lb<1>();
   using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cx<T>* lines = reinterpret_cast<cx<T>*>(smem_raw);
+  cx<T>* tab = reinterpret_cast<cx<T>*>(smem_raw);
+  cx<T>* lines = tab + 2 * M;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int ll = lane / TL, t = lane % TL;
   cx<T>* bl = lines + (warp * LPW + ll) * LB;
   const int ngroups = g.n0 * g.n1 / LPW;
   const int gbase = (blockIdx.x * (blockDim.x >> 5) + warp) * gpw;
-#pragma unroll 1
-  for (int gi = 0; gi < gpw; ++gi) {
-    const int grp = gbase + gi;
-    if (grp >= ngroups) break;
-    const long long line = (long long)grp * LPW + ll;
-    const T* row = in + line * N2;
-    cx<T> v[E], xn;
+  cx<T> v[E], xn;
+  auto load = [&](int grp) {
+    const T* row = in + ((long long)grp * LPW + ll) * N2;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
       const T2 q = *reinterpret_cast<const T2*>(row + 2 * (t + TL * m));
       v[m] = mk<T>(q.x, q.y);
     }
-    xl_forward<T, N2, TW_MAX>(bl, twg, t, xl_mask(), v, v, xn);
+  };
+  if (gbase < ngroups) load(gbase);  // the first rows travel with the table
+  xl_load_tab<T, N2, TW_MAX>(tab, twg);
+  __syncthreads();
+#pragma unroll 1
+  for (int gi = 0; gi < gpw; ++gi) {
+    const int grp = gbase + gi;
+    if (grp >= ngroups) break;
+    const long long line = (long long)grp * LPW + ll;
+    if (gi > 0) load(grp);
+    xl_forward<T, N2, true>(bl, tab, t, xl_mask(), v, v, xn);
     cx<T>* dst = spec + line * g.P;
 #pragma unroll
     for (int m = 0; m < E; ++m) dst[t + TL * m] = v[m];

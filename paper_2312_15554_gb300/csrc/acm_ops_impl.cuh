@@ -133,12 +133,12 @@ static cudaError_t l_x_r2c(const Geo& g, int nprob, int nc, void* spec, long lon
 
 template <typename T, int N2>
 static cudaError_t l_x_r2c_lr(const Geo& g, void* spec, const void* in, const void* tw, cudaStream_t s) {
-  constexpr int smem = xs_smem_bytes<T, N2, 1, 0>();
+  constexpr int smem = xr_smem_bytes<T, N2>();
   static const cudaError_t attr = set_smem(k_x_r2c_lr<T, N2>, smem);
   if (attr != cudaSuccess) return attr;
   const XGrid x = xs_grid(g.n0 * g.n1 / XL<T, N2>::LPW);
-  k_x_r2c_lr<T, N2><<<x.blocks, x.warps * 32, xs_smem_bytes<T, N2, 1, 0>(x.warps), s>>>((cx<T>*)spec, (const T*)in, g,
-                                                                                        (const cx<T>*)tw, x.gpw);
+  k_x_r2c_lr<T, N2><<<x.blocks, x.warps * 32, xr_smem_bytes<T, N2>(x.warps), s>>>((cx<T>*)spec, (const T*)in, g,
+                                                                                  (const cx<T>*)tw, x.gpw);
   return cudaGetLastError();
 }
 

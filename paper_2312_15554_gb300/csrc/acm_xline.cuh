@@ -164,12 +164,20 @@ __device__ __forceinline__ void xl_stage2(const cx<T>* sl, const cx<T>* tw, int 
   });
 }
 
-// The second stage of a forward transform with every twiddle read from the master
-// table W_TWM^k, each a correctly rounded root: the product of a loaded and a
-// compile-time root above is one rounding more per value.
+// The second stage of a forward transform with every twiddle tabulated, each one
+// rounded root (the product of a loaded and a compile-time root above is one rounding
+// more per value). The block's table in shared memory: W_N2^k at k, W_M^{j r} at
+// M + E r + j (0 <= j < E): lanes of a line read consecutive entries, its lines the same.
 template <typename T, int N2, int TWM>
-__device__ __forceinline__ void xl_stage2_tab(const cx<T>* sl, const cx<T>* __restrict__ master, int t,
-                                              cx<T> (&v)[XL<T, N2>::E]) {
+__device__ __forceinline__ void xl_load_tab(cx<T>* tab, const cx<T>* __restrict__ master) {
+  using L = XL<T, N2>;
+  for (int e = threadIdx.x; e < 2 * L::M; e += blockDim.x) {
+    const int q = e - L::M;
+    tab[e] = master[q < 0 ? e * (TWM / N2) : (q / L::E) * (q % L::E) * (TWM / L::M)];
+  }
+}
+template <typename T, int N2>
+__device__ __forceinline__ void xl_stage2_tab(const cx<T>* sl, const cx<T>* tab, int t, cx<T> (&v)[XL<T, N2>::E]) {
   using L = XL<T, N2>;
   constexpr int E = L::E, TL = L::TL, NB = L::NB, M = L::M;
 #pragma unroll
@@ -179,7 +187,7 @@ __device__ __forceinline__ void xl_stage2_tab(const cx<T>* sl, const cx<T>* __re
 #pragma unroll
     for (int r = 0; r < TL; ++r) w2[r] = sl[pad(j + E * r)];
 #pragma unroll
-    for (int r = 1; r < TL; ++r) w2[r] = cmul_fma<0>(w2[r], master[j * r * (TWM / M)]);
+    for (int r = 1; r < TL; ++r) w2[r] = cmul_fma<0>(w2[r], tab[M + E * r + j]);
     dft<TL, -1>(w2);
 #pragma unroll
     for (int r = 0; r < TL; ++r) v[i + NB * r] = w2[r];
@@ -223,8 +231,8 @@ __device__ __forceinline__ void xl_inverse(cx<T>* sl, const cx<T>* tw, int t, un
 // lane (TL - t) mod TL of its line) instead of a second pass through sl.
 // Positions m and E-1-m are finished together; lane 0's partner E - m of
 // position m was overwritten one step earlier and is carried in a register.
-// TWM > 0: tw is the master table W_TWM^k and every twiddle is read from it.
-template <typename T, int N2, int TWM = 0>
+// TAB: tw is the table of xl_load_tab.
+template <typename T, int N2, bool TAB = false>
 __device__ __forceinline__ void xl_forward(cx<T>* sl, const cx<T>* tw, int t, unsigned mask,
                                            cx<T> (&v)[XL<T, N2>::E], cx<T> (&X)[XL<T, N2>::E], cx<T>& xn) {
   using L = XL<T, N2>;
@@ -237,13 +245,13 @@ __device__ __forceinline__ void xl_forward(cx<T>* sl, const cx<T>* tw, int t, un
   for (int r = 0; r < E; ++r) sl[pad(t * E + r)] = v[r];
   if constexpr (TL > 1) {
     __syncwarp(mask);
-    if constexpr (TWM > 0) xl_stage2_tab<T, N2, TWM>(sl, tw, t, v);
+    if constexpr (TAB) xl_stage2_tab<T, N2>(sl, tw, t, v);
     else xl_stage2<T, N2, -1>(sl, tw, t, v);
     __syncwarp(mask);  // the stage-2 reads are done before sl is reused
   }
   auto post = [&](auto P, cx<T> zk, cx<T> zp) {
     constexpr int m = decltype(P)::value;
-    if constexpr (TWM > 0) return xl_post_tab(zk, zp, tw[(t + TL * m) * (TWM / N2)]);
+    if constexpr (TAB) return xl_post_tab(zk, zp, tw[t + TL * m]);
     else if constexpr (L::TAB) return xl_post_tab(zk, zp, tw[L::TW0 + t + TL * m]);
     else return xl_post<m, E>(zk, zp, wt);
   };

@@ -1319,8 +1319,9 @@ acm_status batch_stokes_run(acm_batch* b, const uint8_t* const* H, const acm_sto
 // Tile autotuner: times each candidate tile width of the strided passes of the
 // solver loops on this context's workspace (nprob problems, CUDA events on the
 // context's stream) and keeps the fastest. The tile width only regroups which
-// columns a block transforms, so every choice gives the same fields; only the
-// order of the FP64 partial sums of the z pass changes.
+// columns a block transforms: within the row segments, and within the positive
+// widths, every choice gives the same fields and only the order of the residual
+// partial sums of the z pass changes (FP32 segments round differently from the rest).
 // ---------------------------------------------------------------------------
 struct TuneJob {
   int axis, op, nc;

@@ -1,15 +1,16 @@
-// acm_fft.cuh -- shared-memory Stockham FFT building blocks for sm_103a.
+// acm_fft.cuh -- FFT building blocks for sm_103a: in-register DFTs and roots (all
+// passes), transforms of lines in shared memory (the block-phase x passes; the
+// line-resident x passes and the strided passes keep their lines in registers, see
+// acm_xline.cuh and acm_rpass.cuh), copies, reductions.
 //
-// Every 1D transform of length N runs on one "line" held in shared memory.
-// A line is processed by T = N / E threads of one warp (E = elements per
-// thread, at most 16), so the stages synchronise with __syncwarp only.
-// Each stage reads E values into registers, applies the twiddles and an
-// in-register DFT of radix R (R divides E), and writes the results back in
+// fft_line: a line of length N in shared memory is processed by T = N / E threads of
+// one warp (E = elements per thread, at most 16), so the stages synchronise with
+// __syncwarp only. Each stage reads E values into registers, applies the twiddles
+// and an in-register DFT of radix R (R divides E), and writes the results back in
 // Stockham (self-sorting) order, so the output is in natural order.
 //
 // Shared-memory lines are padded with one slot per 16 elements (pad()) so that
-// the stride-R writes of the first stage and the transposed tile loads of the
-// strided passes spread over all banks.
+// the stride-R writes of the first stage spread over all banks.
 //
 // The forward transform uses exp(-2 pi i k n / N) and is unnormalised; the
 // inverse uses exp(+2 pi i k n / N) and is unnormalised too.
@@ -118,11 +119,9 @@ __host__ __device__ constexpr int ept(int n) { return n < 16 ? n : 16; }  // ele
 // for FP32 complex, 8 for FP64 complex), each touching one slot. When a line's
 // transform uses TL < W threads, a wavefront spans W/TL lines and each line
 // covers TL consecutive slots, so the lines must start TL slots apart modulo W:
-// stride = TL * odd (mod W). When lines are loaded as the TX columns of a tile
-// (TX threads per row, W/TX rows per wavefront) the columns must start W/TX
-// slots apart. The first stride at or above the padded length that meets the
-// active constraint is used; with TL < W the transform's constraint wins (it
-// is accessed more often).
+// stride = TL * odd (mod W), the first at or above the padded length. TX > 0 (in the
+// widths the strided passes report, see tx_ok): with TL >= W, lines that are loaded
+// as the TX columns of a tile start W/TX slots apart.
 __host__ __device__ constexpr int line_stride(int L, int TL, int TX, int W) {
   int ls = (L - 1) + ((L - 1) >> 4) + 1;
   const int q = TL < W ? TL : (TX >= 1 && TX < W ? W / TX : 1);
@@ -417,7 +416,7 @@ __device__ __forceinline__ void fft_line(cx<T>* s, int t, const cx<T>* tw, unsig
 }
 
 // ---------------------------------------------------------------------------
-// asynchronous global -> shared copies (cp.async): the loads of a tile are all
+// asynchronous global -> shared copies (cp.async): the loads of a row are all
 // in flight at once and do not pass through registers
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
@@ -426,13 +425,6 @@ template <int BYTES>
 __device__ __forceinline__ void cp_async(void* smem, const void* gmem) {
   static_assert(BYTES == 4 || BYTES == 8 || BYTES == 16, "cp.async size");
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(smem_u32(smem)), "l"(gmem), "n"(BYTES));
-}
-
-// copy BYTES when pred, else write zeros to shared memory (no global access)
-template <int BYTES>
-__device__ __forceinline__ void cp_async_pred(void* smem, const void* gmem, bool pred) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(smem_u32(smem)), "l"(gmem), "n"(BYTES),
-               "r"(pred ? BYTES : 0));
 }
 
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }

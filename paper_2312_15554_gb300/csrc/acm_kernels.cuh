@@ -9,15 +9,14 @@
 //   stokes_finalize  residuals, tolerances (Eq. 11-12), stop test, Eq. 22
 //   x_stokes_rhs     w and its R2C again where b came out otherwise (and before
 //                    the first iteration)
-//   strided<FWD>     forward FFT along y
-//   strided<STOKES>  forward FFT along z, Eq. 13 solve per wavevector, q update
+//   k_lpass<FWD>     forward FFT along y
+//   k_lpass_z        forward FFT along z, Eq. 13 solve per wavevector, q update
 //                    of Eq. 9 in Fourier space, divergence residuals by
 //                    Parseval, inverse FFT along z
-//   strided<INV>     inverse FFT along y
+//   k_lpass<INV>     inverse FFT along y
 // One solute iteration (Section 3.2) is x_solute (C2R of grad chi, local
-// residual terms of Eq. 18, R2C), strided<FWD>, strided<SOLUTE> (Eq. 20 with
-// the Eq. 21 symbols, Eq. 19 residuals by Parseval), strided<INV> and
-// solute_finalize.
+// residual terms of Eq. 18, R2C), k_lpass_fsol, k_lpass_z (Eq. 20 with the Eq. 21
+// symbols, Eq. 19 residuals by Parseval), k_lpass_isol and solute_finalize.
 //
 // The ADMM state is reduced by an identity of steps 2-3: with a^0 = H lambda^0,
 // step 3 gives a^{n+1} = H lambda^{n+1} after every iteration, so a is never

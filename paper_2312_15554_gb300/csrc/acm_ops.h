@@ -9,7 +9,7 @@
 namespace acm {
 
 // P_FWD_SOL / P_INV_SOL: the y passes of the solute iteration (derivative
-// terms of axis 1 folded in; see the strided kernel); P_SOLUTE: its z pass.
+// terms of axis 1 folded in; see acm_rpass.cuh); P_SOLUTE: its z pass.
 enum PassOp { P_FWD = 0, P_INV = 1, P_INV_SCALE = 2, P_STOKES = 3, P_SOLUTE = 4, P_DERIV = 5, P_FWD_SOL = 6,
               P_INV_SOL = 7 };
 

@@ -8,8 +8,9 @@
 
 namespace acm {
 
-// The default tile width (kx columns) a strided pass reports: about 256 threads
-// over its components, at least 2 columns, at most 64 KB of shared memory.
+// The default tile width (kx columns) a strided pass reports (see tx_ok; it runs the
+// width that lp_width takes from the grid): about 256 threads over its components, at
+// least 2 columns, at most 64 KB of shared memory.
 constexpr int pick_tx(int csize, int N, int NC) {
   int tl = N / ept(N);
   int tx = 16;
@@ -174,8 +175,7 @@ static cudaError_t l_x_c2r(const Geo& g, int nprob, int nc, const void* spec, lo
 
 // Tile choices of a pass (Geo::txs): 0 lets the pass pick its width from the
 // grid; the solver passes at N >= 64 also take -1, 1, 2 (half, double, four
-// times the default width reported, where that number stays within 2..32 columns,
-// 1536 line threads and 200 KB) and, at N = 64, 128 and 256, 3 and 4 (a full and
+// times the default width reported) and, at N = 64, 128 and 256, 3 and 4 (a full and
 // a half 128-byte row segment, reported as -W). FP32 lines of 128 and 256 points also
 // take 5, a quarter segment: what a pass of a small grid picks by itself, so the tuner
 // has to be able to pick it too (z Stokes, us a launch at half and quarter segments:
@@ -187,6 +187,10 @@ constexpr bool tunable() {
                      OP == OP_FWD_SOL || OP == OP_INV_SOL);
 }
 
+// Which positive widths are offered: a list that callers may have saved, so it stays
+// what it was when a tile of TX columns was one block of at most 1536 line threads and
+// 200 KB of shared memory. A pass runs the nearest width it is compiled for
+// (lp_width), so several of them can name one kernel.
 template <typename T, int N, int OP, int NC, int TX>
 constexpr bool tx_ok() {
   return TX >= 2 && TX <= 32 && NC * TX * (N / ept(N)) <= 1536 &&

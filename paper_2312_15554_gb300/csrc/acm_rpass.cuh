@@ -109,9 +109,13 @@ __host__ __device__ constexpr int lp_smem() {
   return lp_groups(OP) * W * LCfg<T, N, W>::BS * (int)sizeof(cx<T>);
 }
 
-// blocks per SM the launch bound asks for: at most 80 registers a thread in FP32
-// (64 in the solute z and y passes, which fit them: z 19 us instead of 23
-// at 128^3), 128 in FP64
+// Blocks per SM the launch bound asks for. FP32: 768 threads an SM, 80 registers a
+// thread (64 at 1024 threads in the solute z and y passes, which fit them: z 19 us
+// instead of 23 at 128^3); FP64: 512 threads, 128 registers. At most 16 blocks are
+// asked for, which leaves one-warp blocks 128 registers, and whole ones: FP64 z Stokes
+// in blocks of 192 or 384 threads may take 168, and at N = 512, 768 threads, 80. The
+// FP32 z operators spill 4 to 12 bytes at 80 registers, the FP64 Stokes ones 32 in
+// blocks of 96 threads at N = 128 and 24 (40 in the plane pass) at 512.
 template <typename T, int N, int OP, int W>
 __host__ __device__ constexpr int lp_minblocks() {
   const int threads = lp_groups(OP) * LCfg<T, N, W>::NT;
@@ -440,7 +444,7 @@ __global__ void __launch_bounds__(LCfg<T, N, W>::NT, (lp_minblocks<T, N, OP, W>(
 // read once its own component has left the registers (with the inputs it would
 // live through the forward transform: spills, 577 us a launch against 544 at
 // 256^3 and three problems). Issue slots bound these passes (40% busy, DRAM at
-// half its rate): two transforms and the operator are about 1900 instructions a
+// half its rate): two transforms and the operator are about 1750 instructions a
 // thread. Against one thread per line holding two components at a time (166
 // registers, 12 warps an SM) z Stokes takes 544 us for 606, z solute 327 for 338
 // in the block-wide tile it used; 512^3 lines, block-wide before, 5.56 ms for 6.56.

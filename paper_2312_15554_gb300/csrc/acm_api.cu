@@ -1860,24 +1860,31 @@ acm_status acm_batch_tiles(acm_batch* b, int cell, int fp64, int tiles[NTUNE]) {
 acm_status acm_batch_history_enable(acm_batch* b, int cap) {
   if (!b || cap < 0) return ACM_ERR_ARG;
   if (b->st) CK(cudaStreamSynchronize(b->st));
-  for (auto& gr : b->groups) {
-    acm_ctx* c = gr.c;
-    if (c->hist_b) cudaFree(c->hist_b);
-    c->hist_b = nullptr;
-    c->hist_b_cap = 0;
-    if (cap > 0) {
-      if (cudaMalloc(&c->hist_b, (size_t)c->B * cap * STOKES_HIST * sizeof(double)) != cudaSuccess) {
-        cudaGetLastError();
-        return ACM_ERR_NOMEM;
-      }
-      c->hist_b_cap = cap;
-    }
-    gr.iters.clear();
-  }
-  // a captured loop holds the old history pointer
+  // a captured loop holds the old history pointer: it goes first, so that it does not
+  // outlive a failed allocation
   if (b->graph.exec) {
     cudaGraphExecDestroy(b->graph.exec);
     b->graph.exec = nullptr;
+  }
+  auto off = [&] {
+    for (auto& gr : b->groups) {
+      if (gr.c->hist_b) cudaFree(gr.c->hist_b);
+      gr.c->hist_b = nullptr;
+      gr.c->hist_b_cap = 0;
+      gr.iters.clear();
+    }
+  };
+  off();
+  for (auto& gr : b->groups) {
+    if (cap == 0) break;
+    acm_ctx* c = gr.c;
+    if (cudaMalloc(&c->hist_b, (size_t)c->B * cap * STOKES_HIST * sizeof(double)) != cudaSuccess) {
+      cudaGetLastError();
+      c->hist_b = nullptr;
+      off();
+      return ACM_ERR_NOMEM;
+    }
+    c->hist_b_cap = cap;
   }
   return ACM_OK;
 }
